@@ -448,101 +448,864 @@ arnoldi_step_kernel(int n, int rows_per_cta, const int* __restrict__ rowptr,
     w[i] = static_cast<T>(static_cast<double>(w[i]) * inv);
 }
 
-// The same FP64 step with w resident on chip.  w = A v_j is first formed in
-// V's column j+1 by the SELL SpMV kernel (full occupancy, and the whole L1
-// for the gathers of v_j); then CTA b of this cooperative kernel loads its
-// rows [b R, (b+1) R) of w into shared memory and keeps them there through
-// the MGS phases to the final normalisation.  A thread always touches the
-// same rows, so w needs no barrier of its own; each phase streams only v_l
-// (just read as the previous phase's v_{l+1}, an L2 hit) and v_{l+1},
-// instead of reading and writing w through HBM as well.  Phase order, fused
-// next-vector dot and per-CTA partials are those of arnoldi_step_kernel;
-// only the rows a CTA owns differ.
-__global__ void __launch_bounds__(kCoopThreads, 1)
-arnoldi_mgs_resident_kernel(int n, int rows_cta, double* __restrict__ V, int64_t ld, int j,
+// The same FP64 step with w resident on chip, in fixed point.  w = A v_j is
+// first formed in V's column j+1 by the SELL SpMV kernel (full occupancy,
+// and the whole L1 for the gathers of v_j); then CTA b of this cooperative
+// kernel loads its rows [b R, (b+1) R) of w into shared memory and keeps
+// them there through the projections to the final normalisation, streaming
+// the vectors past them.
+//
+// In FP64 the FP64 pipe bounds a projection (two FMAs a row at 2 a clock and
+// SM: 13 of 20 us at 4.19M rows, where the vector takes 5 us from HBM), then
+// the exchange of the partial sums between the CTAs (4 us).  So:
+//   * v_l is kept as signed 60-bit integers relative to the largest
+//     magnitude of the CTA's rows of it (|v| < 2^ev), w as integers of at
+//     most 61 bits relative to a bound on its rows (unit 2^(ew - 62)); both
+//     are cut into two signed 32-bit halves, and a row costs seven 32 x 32
+//     bit multiply-adds instead of two FP64 FMAs:
+//       dot:  sum vh wh 2^64 + (vh wl + vl wh) 2^32 + vl wl, exact but for the
+//             low half of vl wl;
+//       w -= h v:  h 2^ev in units of w, rounded to an integer, times v 2^-60,
+//             rounded to w's unit.
+//     The unit of v is 2^-58 of the CTA's largest entry or less, that of w
+//     2^-60 or less at the start: the projections round less than FP64 ones
+//     do.  Since |w| can grow while it is projected, its bound grows by
+//     |h| 2^ev per projection and w is shifted down when the bound reaches
+//     2^61 units.
+//   * the CTAs' partial sums are added with integer atomics on a common grid
+//     of 2^-70 ||A v_j|| (no partial sum exceeds ||A v_j||): any order gives
+//     the same total.  Each of the two words of a sum counts its arrivals in
+//     its low byte, so the sum, its completeness and the release of the
+//     waiters are one L2 round trip (1.2 us, the counter barrier with 152
+//     partial sums read back 3.6 us); no fence is needed, the CTAs share
+//     nothing else.
+//   * the exchange overlaps the next pass over the rows: pass q takes h_q v_q
+//     out of w and sums d_{q+2} = v_{q+2}.w, in which h_{q+1} v_{q+1} is
+//     still present, and h_{q+2} = d_{q+2} - (v_{q+2}.v_{q+1}) h_{q+1}: the
+//     coefficient MGS computes, in another rounding order.  The products of
+//     neighbouring vectors are formed once, when a vector is made.
+// The new vector is w scaled in fixed point, and rounded once to FP64 for the
+// next product with A.  When ||A v_j||^2 is not a normal number well inside FP64's range (zero, an
+// overflow, a NaN in the matrix) the step runs in FP64 on the decoded
+// vectors, one projection per barrier.
+//
+// Measured, whole pre-pass with its products, FP64 pipe -> here: 120 steps
+// at 4.19M rows (25 entries) 172 -> 98 ms (a projection 19.9 -> 8.9 us, 3.8
+// TB/s of the vector's bytes), at 2.10M (7 entries) 93 -> 45 ms; 60 steps at
+// 152K rows 11.1 -> 4.6 ms (5.4 -> 1.9 us: the exchange's latency).  What is
+// left at 4.19M rows is reading v_{q+2} from HBM and, for the rows past the
+// four batches that tensor memory holds, v_q once more through L2.  1024
+// threads (64 registers) were slower at every size (152K rows: 6.0 ms), a
+// ring of four smaller batches as well (144 ms at 4.19M rows), and neither
+// prefetch into L2 (lines or bulk, one to six batches ahead) changed
+// anything.
+constexpr int kFxThreads = 512;   // one CTA per SM; 128 registers hold two batches of loads
+constexpr int kFxBatch = 4;       // pairs of rows per thread and batch of loads
+constexpr int kFxTmem = 4;        // batches that tensor memory keeps, of two vectors
+constexpr int kFxV = 60;          // bits of v below 2^ev
+constexpr int kFxW = 62;          // bits of w below 2^ew (at most 2^61 used)
+constexpr int kFxGrid = 70;       // bits of a partial sum below ||A v_j||
+
+__device__ __forceinline__ double pow2d(int e) {   // 2^e, |e| < 1022
+  return __longlong_as_double(static_cast<long long>(e + 1023) << 52);
+}
+
+// x 2^(bits - e) rounded to the nearest integer, |x| < 2^e, bits <= 62
+// (0 for a non-finite x)
+__device__ __forceinline__ long long to_fixed(double x, int e, int bits) {
+  const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int E = static_cast<int>((u >> 52) & 0x7FF);
+  unsigned long long m = 0;
+  if (E != 0 && E != 0x7FF) {
+    const unsigned long long mant = (u & ((1ull << 52) - 1)) | (1ull << 52);
+    const int sh = E - 1075 + bits - e;   // <= bits - 53
+    if (sh >= 0) m = mant << (sh > 9 ? 9 : sh);
+    else if (sh > -60) m = (mant + (1ull << (-sh - 1))) >> (-sh);
+  }
+  return (u >> 63) ? -static_cast<long long>(m) : static_cast<long long>(m);
+}
+
+// the least e with |x| < 2^e for the bit pattern of a finite |x| > 0
+// (subnormals: -1021)
+__device__ __forceinline__ int exponent_above(unsigned long long bits) {
+  const int E = static_cast<int>((bits >> 52) & 0x7FF);
+  return (E == 0 ? 1 : E) - 1022;
+}
+
+// a signed integer as (high word, signed low word): x = hi 2^32 + lo with
+// |lo| <= 2^31, stored with the high word already corrected
+__device__ __forceinline__ long long fx_code(long long x) {
+  return x + ((x << 1) & 0x100000000ll);
+}
+__device__ __forceinline__ double fx_decode(long long code, double unit) {
+  const long long x = (static_cast<long long>(static_cast<int>(code >> 32)) << 32) +
+                      static_cast<int>(code);
+  return static_cast<double>(x) * unit;
+}
+
+// a b + c.  In PTX: written in C++, the compiler forms a 64 x 64 bit product
+// of halves taken from a 64-bit word (three multiply-adds instead of one).
+__device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+
+// one row's product, v = (vh, vl), w = (wh, wl):
+// hh += vh wh, c += vh wl + vl wh + the high half of vl wl
+__device__ __forceinline__ void fx_mul(int vl, int vh, int wl, int wh, long long& hh, long long& c) {
+  hh = fx_mad(vh, wh, hh);
+  c = fx_mad(vh, wl, c);
+  c = fx_mad(vl, wh, c);
+  c += __mulhi(vl, wl);
+}
+// (high word, signed low word) of x
+__device__ __forceinline__ void fx_split(long long x, int& lo, int& hi) {
+  lo = static_cast<int>(x);
+  hi = static_cast<int>(x >> 32) + static_cast<int>(static_cast<unsigned>(lo) >> 31);
+}
+__device__ __forceinline__ void fx_dot(int vl, int vh, long long w, long long& hh, long long& c) {
+  int wl, wh;
+  fx_split(w, wl, wh);
+  fx_mul(vl, vh, wl, wh, hh, c);
+}
+// c's high half into hh (exact: c keeps the low half); at least every four
+// rows (each adds less than 2^60.6 to |c|)
+__device__ __forceinline__ void fx_flush(long long& hh, long long& c) {
+  hh += c >> 32;
+  c &= 0xFFFFFFFFll;
+}
+
+// w + v (nh 2^32 + nl) 2^-60, rounded (vl nl, at most four units, left out)
+__device__ __forceinline__ long long fx_axpy(int vl, int vh, int nh, int nl, long long w) {
+  const long long c = fx_mad(vl, nh, fx_mad(vh, nl, 1ll << 27));
+  const long long m = fx_mad(vh, nh, 0);
+  return w + (m << 4) + (c >> 28);
+}
+// x (nh 2^32 + nl) 2^-64, rounded, |x| < 2^62
+__device__ __forceinline__ long long fx_scale(long long x, int nh, int nl) {
+  int xl, xh;
+  fx_split(x, xl, xh);
+  long long c = fx_mad(xl, nh, fx_mad(xh, nl, 1ll << 31));
+  c += __mulhi(xl, nl);
+  return fx_mad(xh, nh, c >> 32);
+}
+
+// Tensor memory as storage: this thread's lane, four pairs of rows in 16
+// consecutive columns.
+__device__ __forceinline__ void fx_tmem_st(uint32_t addr, const int4* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+      "%14,%15,%16};" ::"r"(addr),
+      "r"(v[0].x), "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z),
+      "r"(v[1].w), "r"(v[2].x), "r"(v[2].y), "r"(v[2].z), "r"(v[2].w), "r"(v[3].x), "r"(v[3].y),
+      "r"(v[3].z), "r"(v[3].w)
+      : "memory");
+}
+// (the wait is in the same statement: no use of the registers can move
+// before it)
+__device__ __forceinline__ void fx_tmem_ld(uint32_t addr, int4* v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(v[0].x), "=r"(v[0].y), "=r"(v[0].z), "=r"(v[0].w), "=r"(v[1].x), "=r"(v[1].y),
+        "=r"(v[1].z), "=r"(v[1].w), "=r"(v[2].x), "=r"(v[2].y), "=r"(v[2].z), "=r"(v[2].w),
+        "=r"(v[3].x), "=r"(v[3].y), "=r"(v[3].z), "=r"(v[3].w)
+      : "r"(addr)
+      : "memory");
+}
+
+// T 2^s; rounded to the nearest integer for s < 0
+__device__ __forceinline__ __int128 fx_shift(__int128 T, int s) {
+  if (s >= 0) return T << (s > 64 ? 64 : s);
+  const int r = -s > 120 ? 120 : -s;
+  return (T + (static_cast<__int128>(1) << (r - 1))) >> r;
+}
+
+// A coefficient on the common grid: (hi 2^36 + lo) 2^(e0 - 70), 0 <= lo < 2^36
+struct FxCoef {
+  long long hi, lo;
+  __device__ __forceinline__ void carry() {
+    hi += lo >> 36;
+    lo &= (1ll << 36) - 1;
+  }
+  // (hi 2^36 + lo) 2^s rounded, for results below 2^62
+  __device__ __forceinline__ long long scaled(int s) const {
+    if (s >= 0) return s > 26 ? 0 : (hi << (36 + s)) + (lo << s);
+    int r = -s;
+    if (r <= 36) return (hi << (36 - r)) + ((lo + (1ll << (r - 1))) >> r);
+    r -= 36;
+    return (hi + (1ll << ((r > 62 ? 62 : r) - 1))) >> (r > 62 ? 62 : r);
+  }
+  // bits that scaled(s) takes at most
+  __device__ __forceinline__ int bits(int s) const {
+    if (hi == 0 && lo == 0) return 0;
+    const unsigned long long m = static_cast<unsigned long long>(hi < 0 ? -hi : hi) + 1;
+    return 64 - __clzll(static_cast<long long>(m)) + 36 + s;
+  }
+  __device__ __forceinline__ double in_grid() const {
+    return fma(static_cast<double>(hi), 68719476736.0, static_cast<double>(lo));
+  }
+};
+
+// words of one step's exchanges: [0] the full barriers' counter, then a
+// (low, high) pair per coefficient
+__host__ __device__ constexpr int64_t fx_set_words(int k) { return 2 + 2 * (static_cast<int64_t>(k) + 1); }
+
+// What a pre-pass keeps between its steps beside V: exps, per vector and
+// CTA, the exponents ev; gram[l] = v_{l+1}.v_l of the steps before the last
+// one, whose CTA partials are gpart; two sets of exchange words, used in turn
+// (each step clears the next one's).
+struct FxState {
+  double* red;                 // 2 G partial sums
+  double* gpart;               // G
+  double* gram;
+  int* exps;
+  unsigned long long* set;
+  unsigned long long* next_set;
+  int set_words;
+};
+
+__global__ void __launch_bounds__(kFxThreads, 1)
+arnoldi_mgs_resident_kernel(int n, int rows_cta, double* V, int64_t ld, int j, double* xv,
                             double* __restrict__ H, int ldh, double* __restrict__ wn,
-                            double* __restrict__ red, unsigned* ctr, unsigned base, int* err) {
+                            FxState fs, int* err) {
   extern __shared__ __align__(16) unsigned char coop_smem[];
-  double* ws = reinterpret_cast<double*>(coop_smem);
-  const int G = gridDim.x;
-  const int t = threadIdx.x;
-  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * rows_cta;
+  constexpr int T = kFxThreads, W = kFxThreads / 32;
+  __shared__ unsigned wsum[2][4][W];           // a pass's sums, four limbs per warp
+  __shared__ unsigned long long wmax[W];
+  __shared__ uint32_t tmem_base;
+  __shared__ int bc[2][5];                     // of a pass: -h (nl, nh), w's shift; last pass: two
+  long long* ws = reinterpret_cast<long long*>(coop_smem);      // w, fixed point
+  double* wd = reinterpret_cast<double*>(coop_smem);            // w, FP64 (before and after)
+  const int G = gridDim.x, cta = blockIdx.x;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int64_t r0 = static_cast<int64_t>(cta) * rows_cta;
   const int64_t r1 = (r0 + rows_cta < n) ? r0 + rows_cta : n;
   const int nr = r1 > r0 ? static_cast<int>(r1 - r0) : 0;
-  const double* v0 = V + r0;
+  const int np = (nr + 1) >> 1;                // pairs of rows (the last may be half)
   double* w = V + static_cast<int64_t>(j + 1) * ld + r0;
-  double* pWW = red;
-  double* pA = red + G;
-  double* pB = red + 2 * G;
-  // this CTA's rows of w = A v_j, partials of w.w and v_0.w
-  double accw = 0.0, accv = 0.0;
-  for (int i = t; i < nr; i += kCoopThreads) {
-    const double wi = w[i];
-    ws[i] = wi;
-    accw = fma(wi, wi, accw);
-    accv = fma(v0[i], wi, accv);
+  auto col = [&](int l) { return reinterpret_cast<int4*>(V + static_cast<int64_t>(l) * ld + r0); };
+  unsigned* ctr = reinterpret_cast<unsigned*>(fs.set);
+  unsigned target = 0;
+  double* pWW = fs.red;
+  double* pNN = fs.red + G;
+  constexpr unsigned long long kMag = 0x7FFFFFFFFFFFFFFFull;
+  // largest of the threads' values; every thread receives it
+  auto block_max = [&](unsigned long long m) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, off);
+      m = o > m ? o : m;
+    }
+    __syncthreads();
+    if (lane == 0) wmax[warp] = m;
+    __syncthreads();
+    m = wmax[lane % W];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, off);
+      m = o > m ? o : m;
+    }
+    return m;
+  };
+  // the warp's sum of the threads' hh 2^64 + c 2^32 (0 <= c < 2^32) into
+  // wsum[b], in units of 2^40: limbs of 22 bits, the last one signed
+  auto warp_sums = [&](long long hh, long long c, int b) {
+    const unsigned long long lo = (static_cast<unsigned long long>(hh) << 24) |
+                                  static_cast<unsigned long long>(c >> 8);
+    const long long hi = hh >> 40;
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(lo & 0x3FFFFF));
+    const unsigned s1 = __reduce_add_sync(0xffffffffu, static_cast<unsigned>((lo >> 22) & 0x3FFFFF));
+    const unsigned s2 = __reduce_add_sync(
+        0xffffffffu, static_cast<unsigned>((lo >> 44) | (static_cast<unsigned long long>(hi) << 20)) & 0x3FFFFF);
+    const int s3 = __reduce_add_sync(0xffffffffu, static_cast<int>(hi >> 2));
+    if (lane == 0) {
+      wsum[b][0][warp] = s0;
+      wsum[b][1][warp] = s1;
+      wsum[b][2][warp] = s2;
+      wsum[b][3][warp] = static_cast<unsigned>(s3);
+    }
+  };
+  // the CTA's sum of wsum[b] (by one warp, every lane receives it)
+  auto cta_sum = [&](int b) -> __int128 {
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, lane < W ? wsum[b][0][lane] : 0u);
+    const unsigned s1 = __reduce_add_sync(0xffffffffu, lane < W ? wsum[b][1][lane] : 0u);
+    const unsigned s2 = __reduce_add_sync(0xffffffffu, lane < W ? wsum[b][2][lane] : 0u);
+    const int s3 = __reduce_add_sync(0xffffffffu, lane < W ? static_cast<int>(wsum[b][3][lane]) : 0);
+    const __int128 top = static_cast<__int128>((static_cast<long long>(s3) << 22) + s2) << 44;
+    return top + static_cast<long long>((static_cast<unsigned long long>(s1) << 22) + s0);
+  };
+  auto to_double = [](__int128 x) {
+    return fma(static_cast<double>(static_cast<long long>(x >> 48)), 281474976710656.0,
+               static_cast<double>(static_cast<long long>(x & ((static_cast<__int128>(1) << 48) - 1))));
+  };
+
+  // Pair p = (k U + u) T + t of the CTA's rows is thread t's, batch k.  The
+  // first four batches of v_q stay in tensor memory from the pass that reads
+  // it (as v_{q+2} two passes before) to the one that takes it out of w:
+  // the thread's lane, columns 128 (warp / 4) + 32 k + 16 (q % 2) + 4 u.
+  // (The kernel's registers fill an SM, so no other kernel's allocation can
+  // be in the way there.)
+  constexpr int U = kFxBatch;
+  const int nb = np / (U * T);                 // whole batches
+  const int tail = nb * U * T;                 // first pair of the rest
+  const int nbt = (np + U * T - 1) / (U * T);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(&tmem_base))), "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tm = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) +
+                      static_cast<uint32_t>((warp >> 2) * 128);
+
+  if (cta == 0)   // the words of the next step (used two launches ago)
+    for (int i = t; i < fs.set_words; i += T) fs.next_set[i] = 0;
+  if (j == 0) {
+    // v_0 arrives in FP64: to fixed point in place
+    double* q = V + r0;
+    unsigned long long mx = 0;
+    for (int i = t; i < nr; i += T) {
+      const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(q[i])) & kMag;
+      mx = b > mx ? b : mx;
+    }
+    mx = block_max(mx);
+    int ev = mx == 0 ? -100 : exponent_above(mx);
+    if (ev < -100) ev = -100;
+    if (t == 0) fs.exps[cta] = ev;
+    long long* qc = reinterpret_cast<long long*>(q);
+    for (int p = t; p < np; p += T)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = 2 * p + u;
+        qc[i] = i < nr ? fx_code(to_fixed(q[i], ev, kFxV)) : 0;
+      }
+    __syncthreads();
+  }
+  // this CTA's rows of w = A v_j, partial of w.w, largest magnitude
+  double accw = 0.0;
+  unsigned long long mx = 0;
+  for (int p0 = t; p0 < np; p0 += 4 * T) {
+    double2 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int p = p0 + u * T;
+      x[u] = make_double2(0.0, 0.0);
+      if (2 * p + 1 < nr) x[u] = __ldcg(reinterpret_cast<const double2*>(w) + p);
+      else if (2 * p < nr) x[u].x = w[2 * p];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int p = p0 + u * T;
+      if (p < np) *reinterpret_cast<double2*>(wd + 2 * p) = x[u];
+      accw = fma(x[u].x, x[u].x, accw);
+      accw = fma(x[u].y, x[u].y, accw);
+      unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x[u].x)) & kMag;
+      mx = b > mx ? b : mx;
+      b = static_cast<unsigned long long>(__double_as_longlong(x[u].y)) & kMag;
+      mx = b > mx ? b : mx;
+    }
   }
   {
-    const double sw = block_sum_few_d<kCoopThreads>(accw);
-    const double sv = block_sum_few_d<kCoopThreads>(accv);
-    if (t == 0) { pWW[blockIdx.x] = sw; pA[blockIdx.x] = sv; }
+    const double sw = block_sum_few_d<T>(accw);
+    if (t == 0) pWW[cta] = sw;
   }
-  unsigned target = base + static_cast<unsigned>(G);
+  mx = block_max(mx);
+  // v_j.v_{j-1}, from the partial sums the previous step left
+  const double gnew = j > 0 ? sum_partials_few_d<T>(fs.gpart, G) : 0.0;
+  if (cta == 0 && t == 0 && j > 0) fs.gram[j - 1] = gnew;
+  target += static_cast<unsigned>(G);
   grid_barrier_count(ctr, target, err);
-  if (blockIdx.x == 0) {
-    const double ww = sum_partials_few_d<kCoopThreads>(pWW, G);
-    if (t == 0) wn[j] = sqrt(ww);
-  }
-  // MGS phases l = 0..j: h_l from the previous phase's partials, w -= h_l
-  // v_l, partials of v_{l+1}.w (of w.w in the last phase)
-  double* pin = pA;
-  double* pout = pB;
-  for (int l = 0; l <= j; ++l) {
-    const double h = sum_partials_few_d<kCoopThreads>(pin, G);
-    if (blockIdx.x == 0 && t == 0) H[l + static_cast<int64_t>(j) * ldh] = h;
-    const double* vl = V + static_cast<int64_t>(l) * ld + r0;
-    const double* vn = V + static_cast<int64_t>(l + 1) * ld + r0;
-    double acc = 0.0;
-    int i = t;
-    if (l < j) {
-      for (; i + 3 * kCoopThreads < nr; i += 4 * kCoopThreads) {
-        double wv[4], vv[4], nv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          wv[u] = ws[i + u * kCoopThreads];
-          vv[u] = vl[i + u * kCoopThreads];
-          nv[u] = vn[i + u * kCoopThreads];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const double wi = fma(-h, vv[u], wv[u]);
-          ws[i + u * kCoopThreads] = wi;
-          acc = fma(nv[u], wi, acc);
+  const double ww = sum_partials_few_d<T>(pWW, G);
+  const double wnorm = sqrt(ww);
+  if (cta == 0 && t == 0) wn[j] = wnorm;
+
+  double acc = 0.0;         // FP64 form: thread partial of ||w||^2 after the projections
+  double unit = 0.0;        // fixed point: w's unit then (0: FP64 form)
+  const int evj = fs.exps[static_cast<int64_t>(j) * G + cta];
+  if (ww > 1e-280 && ww < 1e280) {
+    // ------------------------------------------------- fixed point
+    const int e0 = exponent_above(static_cast<unsigned long long>(__double_as_longlong(wnorm)));
+    int ew = mx == 0 ? e0 - 100 : exponent_above(mx) + 2;
+    if (ew < e0 - 100) ew = e0 - 100;
+    long long bound = mx == 0 ? 0 : 1ll << 60;   // |w| <= bound <= 2^61, in units (warp 1 keeps it)
+    auto ev_of = [&](int l) { return fs.exps[static_cast<int64_t>(l) * G + cta]; };
+    // warp 0: adds the CTA's sum of v_l.w in wsum[b] to coefficient l
+    auto post = [&](int l, int b, int evl) {
+      const __int128 P = fx_shift(cta_sum(b), 40 + (ew - kFxW) + (evl - kFxV) + kFxGrid - e0);
+      if (lane < 2) {
+        const unsigned long long part = lane == 0
+            ? static_cast<unsigned long long>(P) & ((1ull << 36) - 1)
+            : static_cast<unsigned long long>(static_cast<long long>(P >> 36));
+        atomicAdd(fs.set + 2 + 2 * l + lane, (part << 8) + 1ull);
+      }
+    };
+    // warp 1: coefficient l once every CTA has posted it
+    auto fetch = [&](int l) -> FxCoef {
+      unsigned long long word = 0;
+      if (lane < 2) {
+        const unsigned long long* slot = fs.set + 2 + 2 * l + lane;
+        const uint64_t t0 = now_ns();
+        unsigned spins = 0;
+        for (;;) {
+          asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(slot) : "memory");
+          if (static_cast<unsigned>(word & 0xFF) == static_cast<unsigned>(G)) break;
+          if ((++spins & 255u) == 0) {
+            // (after a timeout anywhere every wait is left at once)
+            if (*reinterpret_cast<volatile int*>(err) != 0) break;
+            if (now_ns() - t0 > kBarrierNs) {
+              atomicExch(err, 1);
+              break;
+            }
+          }
         }
       }
-      for (; i < nr; i += kCoopThreads) {
-        const double wi = fma(-h, vl[i], ws[i]);
-        ws[i] = wi;
-        acc = fma(vn[i], wi, acc);
+      __syncwarp();
+      FxCoef c;
+      c.lo = static_cast<long long>(__shfl_sync(0xffffffffu, word, 0)) >> 8;
+      c.hi = static_cast<long long>(__shfl_sync(0xffffffffu, word, 1)) >> 8;
+      return c;
+    };
+    // g h: the neighbour's part of a coefficient
+    auto neighbour = [&](double g, const FxCoef& h) -> FxCoef {
+      const double d = g * h.in_grid();
+      const double dh = floor(d * pow2d(-36));
+      FxCoef c;
+      c.hi = static_cast<long long>(dh);
+      c.lo = __double2ll_rn(fma(dh, -68719476736.0, d));
+      return c;
+    };
+    auto minus = [&](const FxCoef& c, const FxCoef& d) -> FxCoef {
+      FxCoef r;
+      r.hi = c.hi - d.hi;
+      r.lo = c.lo - d.lo;
+      r.carry();
+      return r;
+    };
+    // the shift of w that h v needs room for (into ew and bound)
+    auto make_room = [&](const FxCoef& h, int ev, int& e, long long& bd) -> int {
+      const int s = e0 + ev - e + kFxW - kFxGrid;
+      int up = h.bits(s) - 61;
+      long long grow = 0;
+      if (up <= 0) {
+        const long long q = h.scaled(s);
+        grow = q < 0 ? -q : q;                  // |h| 2^ev in units of w
+        up = bd + grow + 8 > (1ll << 61) ? 2 : 0;
+      } else {
+        up += 2;
       }
-    } else {
-      for (; i < nr; i += kCoopThreads) {
-        const double wi = fma(-h, vl[i], ws[i]);
-        ws[i] = wi;
-        acc = fma(wi, wi, acc);
+      if (up > 0) {
+        bd = up < 62 ? (bd >> up) + 1 : 1;
+        const long long q = h.scaled(s - up);
+        grow = q < 0 ? -q : q;
+        e += up;
+      }
+      bd += grow + 8;
+      return up;
+    };
+    // -h 2^ev in units of w, as (nl, nh)
+    auto factor = [&](const FxCoef& h, int ev, int e, int* out) {
+      const long long q = -h.scaled(e0 + ev - e + kFxW - kFxGrid);
+      const int nl = static_cast<int>(q);
+      out[0] = nl;
+      out[1] = static_cast<int>((q - nl) >> 32);
+    };
+    auto shift_w = [&](int up) {
+      const int sh = up > 62 ? 62 : up;
+      for (int p = t; p < np; p += T) {
+        longlong2 f = *reinterpret_cast<longlong2*>(ws + 2 * p);
+        f.x = (f.x + (1ll << (sh - 1))) >> sh;
+        f.y = (f.y + (1ll << (sh - 1))) >> sh;
+        *reinterpret_cast<longlong2*>(ws + 2 * p) = f;
+      }
+    };
+    auto put_h = [&](int l, const FxCoef& h) {
+      if (cta == 0 && lane == 0) H[l + static_cast<int64_t>(j) * ldh] = h.in_grid() * pow2d(e0 - kFxGrid);
+    };
+
+    // w to fixed point; v_0.w and v_1.w
+    {
+      long long h0 = 0, h1 = 0, c = 0, d = 0;
+      const int4* v0 = col(0);
+      const int4* v1 = col(j > 0 ? 1 : 0);
+      for (int k = 0; k < nbt; ++k) {
+        int4 a[U], b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int p = (k * U + u) * T + t;
+          a[u] = b[u] = make_int4(0, 0, 0, 0);
+          if (p < np) {
+            a[u] = __ldcg(v0 + p);
+            b[u] = __ldcg(v1 + p);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int p = (k * U + u) * T + t;
+          if (p < np) {
+            const double2 x = *reinterpret_cast<const double2*>(wd + 2 * p);
+            longlong2 f;
+            f.x = to_fixed(x.x, ew, kFxW);
+            f.y = to_fixed(x.y, ew, kFxW);
+            *reinterpret_cast<longlong2*>(ws + 2 * p) = f;
+            fx_dot(a[u].x, a[u].y, f.x, h0, c);
+            fx_dot(a[u].z, a[u].w, f.y, h0, c);
+            fx_dot(b[u].x, b[u].y, f.x, h1, d);
+            fx_dot(b[u].z, b[u].w, f.y, h1, d);
+            fx_flush(h0, c);
+            fx_flush(h1, d);
+          }
+        }
+        if (k < kFxTmem) {
+          __syncwarp();
+          fx_tmem_st(tm + 32 * k, a);
+          fx_tmem_st(tm + 32 * k + 16, b);
+        }
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      warp_sums(h0, c, 0);
+      warp_sums(h1, d, 1);
+    }
+    int4 a[U], v[U];                   // the next batch of v_q (past tensor memory's) and v_{q+2}
+    const int4* va = nullptr;
+    const int4* vb = nullptr;
+    auto load = [&](int k) {
+      if (k < nb) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = __ldcg(vb + (k * U + u) * T);
+        if (k >= kFxTmem) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) a[u] = __ldcg(va + (k * U + u) * T);
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          a[u] = v[u] = make_int4(0, 0, 0, 0);
+          if (tail + u * T + t < np) {
+            v[u] = __ldcg(vb + tail + u * T);
+            if (k >= kFxTmem) a[u] = __ldcg(va + tail + u * T);
+          }
+        }
+      }
+    };
+    // the first batch of pass q: in flight during the exchange before it
+    auto load_first = [&](int q) {
+      va = col(q) + t;
+      vb = col(q + 2) + t;
+      load(0);
+    };
+    if (j >= 2) load_first(0);
+    __syncthreads();
+    FxCoef hp{}, hc{};                 // warp 1: the last coefficients, h_{q} and h_{q+1}
+    int evp = 0, evc = 0;
+    if (warp == 0) {
+      post(0, 0, ev_of(0));
+      if (j > 0) post(1, 1, ev_of(1));
+    } else if (warp == 1) {
+      evc = ev_of(0);
+      hc = fetch(0);
+      hc.carry();
+      if (j > 1) {
+        const int up = make_room(hc, evc, ew, bound);
+        if (lane == 0) bc[0][2] = up;
+        int f[2];
+        factor(hc, evc, ew, f);
+        if (lane == 0) { bc[0][0] = f[0]; bc[0][1] = f[1]; }
+        ew -= up;                      // (every thread adds it at the pass)
       }
     }
-    const double tot = block_sum_few_d<kCoopThreads>(acc);
-    if (t == 0) pout[blockIdx.x] = tot;
+    __syncthreads();
+
+    // pass q = 0..j-2: w -= h_q v_q, and the sum of v_{q+2}.w
+    for (int q = 0; q + 2 <= j; ++q) {
+      const int b = q & 1;
+      const uint32_t tq = tm + 16 * b;
+      int evn = 0;
+      FxCoef near{};
+      if (warp == 0) {
+        if (q > 0) post(q + 1, b ^ 1, ev_of(q + 1));
+      } else if (warp == 1) {
+        // (FP64, a few hundred cycles: here, not while the others wait)
+        evn = ev_of(q + 1);
+        near = neighbour(fs.gram[q], hc);
+        put_h(q, hc);
+      }
+      const int nl = bc[b][0], nh = bc[b][1], up = bc[b][2];
+      if (up > 0) {
+        shift_w(up);
+        ew += up;
+      }
+      long long hh = 0, c = 0;
+      for (int k = 0; k < nb; ++k) {
+        int4 x[U], y[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) { x[u] = a[u]; y[u] = v[u]; }
+        load(k + 1);
+        if (k < kFxTmem) fx_tmem_ld(tq + 32 * k, x);
+        longlong2* wp = reinterpret_cast<longlong2*>(ws) + k * U * T + t;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          longlong2 f = wp[u * T];
+          f.x = fx_axpy(x[u].x, x[u].y, nh, nl, f.x);
+          f.y = fx_axpy(x[u].z, x[u].w, nh, nl, f.y);
+          wp[u * T] = f;
+          fx_dot(y[u].x, y[u].y, f.x, hh, c);
+          fx_dot(y[u].z, y[u].w, f.y, hh, c);
+          if (u & 1) fx_flush(hh, c);
+        }
+        if (k < kFxTmem) fx_tmem_st(tq + 32 * k, y);
+      }
+      if (nb < nbt && nb < kFxTmem) {
+        __syncwarp();
+        fx_tmem_ld(tq + 32 * nb, a);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int p = tail + u * T + t;
+        if (p < np) {
+          longlong2 f = *reinterpret_cast<const longlong2*>(ws + 2 * p);
+          f.x = fx_axpy(a[u].x, a[u].y, nh, nl, f.x);
+          f.y = fx_axpy(a[u].z, a[u].w, nh, nl, f.y);
+          *reinterpret_cast<longlong2*>(ws + 2 * p) = f;
+          fx_dot(v[u].x, v[u].y, f.x, hh, c);
+          fx_dot(v[u].z, v[u].w, f.y, hh, c);
+          fx_flush(hh, c);
+        }
+      }
+      __syncwarp();
+      if (nb < nbt && nb < kFxTmem) fx_tmem_st(tq + 32 * nb, v);
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      if (q + 3 <= j) load_first(q + 1);
+      warp_sums(hh, c, b);
+      if (warp == 1) {
+        // h_{q+1}, posted a pass ago, and what the next pass needs of it
+        hp = hc;
+        evp = evc;
+        hc = minus(fetch(q + 1), near);
+        evc = evn;
+        if (q + 3 <= j) {
+          const int up2 = make_room(hc, evc, ew, bound);
+          int f[2];
+          factor(hc, evc, ew, f);
+          if (lane == 0) { bc[b ^ 1][0] = f[0]; bc[b ^ 1][1] = f[1]; bc[b ^ 1][2] = up2; }
+          ew -= up2;
+        }
+      }
+      __syncthreads();
+    }
+    // the last coefficient, then the last two projections together
+    if (warp == 0) {
+      if (j > 1) post(j, j & 1, evj);
+    } else if (warp == 1) {
+      int f[4] = {0, 0, 0, 0}, up = 0;
+      if (j > 0) {
+        const FxCoef near = neighbour(gnew, hc);
+        hp = hc;
+        evp = evc;
+        hc = minus(fetch(j), near);
+        evc = evj;
+        up = make_room(hp, evp, ew, bound);
+      }
+      up += make_room(hc, evc, ew, bound);
+      if (j > 0) factor(hp, evp, ew, f);
+      factor(hc, evc, ew, f + 2);
+      ew -= up;
+      if (lane == 0) {
+        for (int i = 0; i < 4; ++i) bc[0][i] = f[i];
+        bc[0][4] = up;
+      }
+      if (j > 0) put_h(j - 1, hp);
+      put_h(j, hc);
+    }
+    __syncthreads();
+    {
+      const int nl = bc[0][0], nh = bc[0][1], ml = bc[0][2], mh = bc[0][3], up = bc[0][4];
+      if (up > 0) {
+        shift_w(up);
+        ew += up;
+      }
+      const int4* va = col(j > 0 ? j - 1 : 0);
+      const int4* vb = col(j);
+      unit = pow2d(ew - kFxW);
+      long long hh = 0, c = 0;
+      unsigned long long m = 0;
+      for (int k = 0; k < nbt; ++k) {
+        int4 x[U], y[U];
+        if (k < kFxTmem) {
+          __syncwarp();
+          fx_tmem_ld(tm + 32 * k + 16 * ((j + 1) & 1), x);
+          fx_tmem_ld(tm + 32 * k + 16 * (j & 1), y);
+        } else {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int p = (k * U + u) * T + t;
+            x[u] = y[u] = make_int4(0, 0, 0, 0);
+            if (p < np) {
+              x[u] = __ldcg(va + p);
+              y[u] = __ldcg(vb + p);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int p = (k * U + u) * T + t;
+          if (p < np) {
+            longlong2 f = *reinterpret_cast<const longlong2*>(ws + 2 * p);
+            f.x = fx_axpy(x[u].x, x[u].y, nh, nl, f.x);
+            f.y = fx_axpy(x[u].z, x[u].w, nh, nl, f.y);
+            f.x = fx_axpy(y[u].x, y[u].y, mh, ml, f.x);
+            f.y = fx_axpy(y[u].z, y[u].w, mh, ml, f.y);
+            *reinterpret_cast<longlong2*>(ws + 2 * p) = f;
+            // w.w in units of 16 unit^2 (|w| may reach 2^61), the largest |w|
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const long long z = i == 0 ? f.x : f.y;
+              int zl, zh;
+              fx_split((z + 2) >> 2, zl, zh);
+              hh = fx_mad(zh, zh, hh);
+              c = fx_mad(2 * zh, zl, c);
+              c += __mulhi(zl, zl);
+              const unsigned long long az = static_cast<unsigned long long>(z < 0 ? -z : z);
+              m = az > m ? az : m;
+            }
+            fx_flush(hh, c);
+          }
+        }
+      }
+      warp_sums(hh, c, 0);
+      mx = block_max(m);               // (its barriers cover wsum)
+    }
+  } else {
+    // -------------------------------------------------- FP64, decoded vectors
+    double* pA = fs.red;            // (free again once every CTA has read pWW)
+    double* pB = fs.red + G;
+    auto unit_of = [&](int l) { return pow2d(fs.exps[static_cast<int64_t>(l) * G + cta] - kFxV); };
+    __syncthreads();
+    const long long* v0 = reinterpret_cast<const long long*>(col(0));
+    double part = 0.0, ul = unit_of(0);
+    for (int i = t; i < nr; i += T) part = fma(fx_decode(v0[i], ul), wd[i], part);
     target += static_cast<unsigned>(G);
     grid_barrier_count(ctr, target, err);
-    double* tmp = pin; pin = pout; pout = tmp;
+    for (int l = 0; l <= j; ++l) {
+      const double tot = block_sum_few_d<T>(part);
+      if (t == 0) pA[cta] = tot;
+      target += static_cast<unsigned>(G);
+      grid_barrier_count(ctr, target, err);
+      const double h = sum_partials_few_d<T>(pA, G);
+      if (cta == 0 && t == 0) H[l + static_cast<int64_t>(j) * ldh] = h;
+      const long long* vl = reinterpret_cast<const long long*>(col(l));
+      const long long* vn = reinterpret_cast<const long long*>(col(l < j ? l + 1 : l));
+      const double un = unit_of(l < j ? l + 1 : l);
+      part = 0.0;
+      for (int i = t; i < nr; i += T) {
+        const double wi = fma(-h, fx_decode(vl[i], ul), wd[i]);
+        wd[i] = wi;
+        part = fma(l < j ? fx_decode(vn[i], un) : wi, wi, part);
+      }
+      ul = un;
+      double* tmp = pA; pA = pB; pB = tmp;
+    }
+    acc = part;
+    pNN = pA;                       // (the other one may still be being read)
   }
-  // normalise into V's column j+1
-  const double nrm = sqrt(sum_partials_few_d<kCoopThreads>(pin, G));
-  if (blockIdx.x == 0 && t == 0) H[(j + 1) + static_cast<int64_t>(j) * ldh] = nrm;
+  if (unit != 0.0) {
+    if (warp == 0) {
+      const __int128 x = cta_sum(0);
+      if (lane == 0) pNN[cta] = to_double(x) * pow2d(40 + 4) * unit * unit;
+    }
+  } else {
+    const double tot = block_sum_few_d<T>(acc);
+    if (t == 0) pNN[cta] = tot;
+  }
+  target += static_cast<unsigned>(G);
+  grid_barrier_count(ctr, target, err);
+  // normalise: fixed point into column j+1, FP64 for the next product with A
+  const double nrm = sqrt(sum_partials_few_d<T>(pNN, G));
+  if (cta == 0 && t == 0) H[(j + 1) + static_cast<int64_t>(j) * ldh] = nrm;
   const double inv = 1.0 / nrm;
-  for (int i = t; i < nr; i += kCoopThreads) w[i] = ws[i] * inv;
+  int ev = -100, sh = 0, nl = 0, nh = 0;
+  if (unit != 0.0) {
+    if (mx != 0) {
+      // v = w unit inv: w shifted left to 62 bits times a 62-bit factor,
+      // |v| < 2^ev with ev as small as the factor's range allows
+      sh = __clzll(static_cast<long long>(mx)) - 2;      // 2^61 <= |w| 2^sh < 2^62 for the largest
+      const double f = unit * inv;                       // v per unit of w
+      ev = exponent_above(static_cast<unsigned long long>(__double_as_longlong(f))) + 62 - sh;
+      if (ev < -100) ev = -100;
+      if (ev > 100) ev = 100;                            // (breakdown: f is not finite)
+      // the factor is f 2^-sh 2^(60 - ev) 2^64 < 2^62
+      const long long q = __double2ll_rn(f * pow2d(64 + kFxV - ev - sh));
+      nl = static_cast<int>(q);
+      nh = static_cast<int>((q - nl) >> 32);
+    }
+  } else {
+    mx = 0;
+    for (int p = t; p < np; p += T) {
+      double2 x = *reinterpret_cast<const double2*>(wd + 2 * p);
+      x.x *= inv;
+      x.y = 2 * p + 1 < nr ? x.y * inv : 0.0;
+      *reinterpret_cast<double2*>(wd + 2 * p) = x;
+      unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x.x)) & kMag;
+      mx = b > mx ? b : mx;
+      b = static_cast<unsigned long long>(__double_as_longlong(x.y)) & kMag;
+      mx = b > mx ? b : mx;
+    }
+    mx = block_max(mx);
+    if (mx != 0) ev = exponent_above(mx);
+    if (ev < -100) ev = -100;
+    if (ev > 100) ev = 100;     // (not a unit vector: the step broke down)
+  }
+  if (t == 0) fs.exps[static_cast<int64_t>(j + 1) * G + cta] = ev;
+  // the new vector, and its product with v_j
+  long long hh = 0, c = 0;
+  longlong2* wc = reinterpret_cast<longlong2*>(w);
+  double* xr = xv + r0;
+  const int4* vj = col(j);
+  const double uv = pow2d(ev - kFxV);
+#pragma unroll 4
+  for (int p = t; p < np; p += T) {
+    const int4 y = __ldcg(vj + p);
+    longlong2 f;
+    double2 x;
+    if (unit != 0.0) {
+      f = *reinterpret_cast<const longlong2*>(ws + 2 * p);
+      f.x = fx_scale(f.x << sh, nh, nl);
+      f.y = fx_scale(f.y << sh, nh, nl);
+      x.x = static_cast<double>(f.x) * uv;
+      x.y = static_cast<double>(f.y) * uv;
+      if (!(inv < HUGE_VAL)) x.x = x.y = inv * 0.0;   // (w vanished: NaN, as 0 / 0)
+    } else {
+      x = *reinterpret_cast<const double2*>(wd + 2 * p);
+      f.x = to_fixed(x.x, ev, kFxV);
+      f.y = to_fixed(x.y, ev, kFxV);
+    }
+    if (2 * p + 1 < nr) *reinterpret_cast<double2*>(xr + 2 * p) = x;
+    else xr[2 * p] = x.x;
+    f.x = fx_code(f.x);
+    f.y = fx_code(f.y);
+    wc[p] = f;
+    fx_mul(y.x, y.y, static_cast<int>(f.x), static_cast<int>(f.x >> 32), hh, c);
+    fx_mul(y.z, y.w, static_cast<int>(f.y), static_cast<int>(f.y >> 32), hh, c);
+    fx_flush(hh, c);
+  }
+  warp_sums(hh, c, 1);
+  __syncthreads();
+  if (warp == 0) {
+    const __int128 x = cta_sum(1);
+    if (lane == 0) fs.gpart[cta] = to_double(x) * pow2d(40 + ev - kFxV + evj - kFxV);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512)
+                 : "memory");
+  }
 }
 
 // FP32 form of the same step with grouped lookahead (used for the steps
@@ -1045,7 +1808,7 @@ bool launch_arnoldi_icwy(const DevCsr& A, const float* val, float* V, int64_t ld
 // Rows per CTA of the resident FP64 step for n rows, or 0 when a CTA's
 // slice of w would not fit in shared memory next to the kernel's static
 // reduction buffers (then the streaming step runs).  One CTA per SM, at
-// least 2048 rows per CTA (fewer CTAs, cheaper barriers, on small systems).
+// least 1024 rows per CTA (fewer CTAs, cheaper exchanges, on small systems).
 int resident_rows_per_cta(int64_t n, int* grid) {
   static std::mutex mu;
   static std::map<int, int> limit;   // device -> dynamic bytes available
@@ -1065,41 +1828,53 @@ int resident_rows_per_cta(int64_t n, int* grid) {
   }
   const int64_t sms = device_sm_count();
   int64_t R = (n + sms - 1) / sms;
-  if (R < 2048) R = 2048;
+  if (R < 1024) R = 1024;
   R = (R + 31) / 32 * 32;
   if (R * static_cast<int64_t>(sizeof(double)) > avail) return 0;
   *grid = static_cast<int>((n + R - 1) / R);
   return static_cast<int>(R);
 }
 
+// doubles of `red` that the resident FP64 step takes in a pre-pass of k steps
+int64_t fixed_red_doubles(int G, int k) {
+  return 3 * static_cast<int64_t>(G) + (k + 1) + (static_cast<int64_t>(k) + 2) / 2 * G +
+         2 * fx_set_words(k);
+}
+
 template <typename T, bool SELL>
 void launch_arnoldi_step(const DevCsr& A, const T* val, T* V, int64_t ld, int j,
-                         double* H, int ldh, double* wn, double* red, int red_cap,
+                         int k, T* xv, double* H, int ldh, double* wn, double* red, int red_cap,
                          unsigned* bar, int* err, cudaStream_t st) {
   if constexpr (sizeof(T) == 8 && SELL) {
     int G = 0;
     const int R = resident_rows_per_cta(A.n, &G);
-    if (R > 0 && G <= device_sm_count() && 3 * G <= red_cap) {
+    if (R > 0 && G <= device_sm_count() && G < 256 && xv && fixed_red_doubles(G, k) <= red_cap) {
       const void* fn = reinterpret_cast<const void*>(arnoldi_mgs_resident_kernel);
       const int smem = R * static_cast<int>(sizeof(double));
       ensure_dynamic_smem(fn, smem);
       int per_sm = 0;
-      SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kCoopThreads, smem));
+      SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kFxThreads, smem));
       if (per_sm >= 1) {
-        // w = A v_j into V's column j+1, then the MGS phases on chip
-        dispatch<0, false, T>(A, A.val, val, V + static_cast<int64_t>(j) * ld, nullptr,
+        const int64_t sw = fx_set_words(k);
+        unsigned long long* sets =
+            reinterpret_cast<unsigned long long*>(red + fixed_red_doubles(G, k) - 2 * sw);
+        FxState fs{};
+        fs.red = red;
+        fs.gpart = red + 2 * G;
+        fs.gram = red + 3 * G;
+        fs.exps = reinterpret_cast<int*>(fs.gram + (k + 1));
+        fs.set = sets + (j & 1) * sw;
+        fs.next_set = sets + ((j + 1) & 1) * sw;
+        fs.set_words = static_cast<int>(sw);
+        if (j == 0) SG_CUDA(cudaMemsetAsync(sets, 0, sizeof(unsigned long long) * 2 * sw, st));
+        // w = A v_j into V's column j+1 (v_j in FP64: V's column 0, then xv),
+        // then the projections on chip
+        dispatch<0, false, T>(A, A.val, val, j == 0 ? V : xv, nullptr,
                               V + static_cast<int64_t>(j + 1) * ld, T(0), T(0), T(1), st);
-        // barriers per step j: one after the w partials, one per MGS phase
-        // (j + 1); the counter (word 16 of the barrier block, zeroed at the
-        // start of the pre-pass) has seen G (j' + 2) arrivals per earlier step
         int n = A.n;
         int rc = R;
-        unsigned* ctr = bar + 16;
-        unsigned base = static_cast<unsigned>(G) * static_cast<unsigned>(j) *
-                        static_cast<unsigned>(j + 3) / 2u;
-        void* args[] = {&n, &rc, &V, &ld, &j, &H, const_cast<int*>(&ldh), &wn, &red, &ctr,
-                        &base, &err};
-        SG_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kCoopThreads), args, smem, st));
+        void* args[] = {&n, &rc, &V, &ld, &j, &xv, &H, const_cast<int*>(&ldh), &wn, &fs, &err};
+        SG_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kFxThreads), args, smem, st));
         count_launch();
         return;
       }
@@ -1545,24 +2320,29 @@ void diag_apply(int64_t n, const double* d, const double* x, double* y, bool div
   SG_LAUNCH_CHECK();
 }
 
-int64_t prepass_red_doubles() { return ic_red_doubles(device_sm_count()); }
+int64_t prepass_red_doubles(int k) {
+  const int64_t a = ic_red_doubles(device_sm_count());
+  const int64_t b = fixed_red_doubles(device_sm_count(), k);
+  return a > b ? a : b;
+}
 
-void arnoldi_step(const DevCsr& A, double* V, int64_t ld, int j, double* H,
+void arnoldi_step(const DevCsr& A, double* V, int64_t ld, int j, int k, double* xv, double* H,
                   int ldh, double* wn, double* red, int red_cap, unsigned* bar,
                   int* err, cudaStream_t st) {
   if (A.sptr && A.sval)
-    launch_arnoldi_step<double, true>(A, A.sval, V, ld, j, H, ldh, wn, red, red_cap, bar, err, st);
+    launch_arnoldi_step<double, true>(A, A.sval, V, ld, j, k, xv, H, ldh, wn, red, red_cap, bar, err, st);
   else
-    launch_arnoldi_step<double, false>(A, A.val, V, ld, j, H, ldh, wn, red, red_cap, bar, err, st);
+    launch_arnoldi_step<double, false>(A, A.val, V, ld, j, k, xv, H, ldh, wn, red, red_cap, bar, err, st);
 }
 
 void arnoldi_step32(const DevCsr& A, float* V, int64_t ld, int j, double* H,
                     int ldh, double* wn, double* red, int red_cap, unsigned* bar,
                     int* err, cudaStream_t st) {
+  float* none = nullptr;
   if (A.sptr && A.sval32)
-    launch_arnoldi_step<float, true>(A, A.sval32, V, ld, j, H, ldh, wn, red, red_cap, bar, err, st);
+    launch_arnoldi_step<float, true>(A, A.sval32, V, ld, j, 0, none, H, ldh, wn, red, red_cap, bar, err, st);
   else
-    launch_arnoldi_step<float, false>(A, A.val32, V, ld, j, H, ldh, wn, red, red_cap, bar, err, st);
+    launch_arnoldi_step<float, false>(A, A.val32, V, ld, j, 0, none, H, ldh, wn, red, red_cap, bar, err, st);
 }
 
 }  // namespace sg

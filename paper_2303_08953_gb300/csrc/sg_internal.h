@@ -93,19 +93,23 @@ void spmv_newton32(const DevCsr& A, const float* x, const float* z, float* y,
                    float theta, float c, float gamma, cudaStream_t st);
 // One Arnoldi step of the Ritz pre-pass (cooperative launch): V[:, j+1] =
 // normalised MGS projection of A V[:, j]; writes H(0..j+1, j) (ld ldh) and
-// wn[j] = ||A v_j||.  red: >= 3 x SMs doubles (FP64); bar: 64 zeroed unsigned
-// words (barrier state); err: set to 1 if a barrier wait ran out.
-void arnoldi_step(const DevCsr& A, double* V, int64_t ld, int j, double* H,
+// wn[j] = ||A v_j||.  k: steps of the whole pre-pass (0..k-1, run in order on
+// one V, xv and red); red: >= prepass_red_doubles(k) doubles; bar: 64 zeroed
+// unsigned words (barrier state); err: set to 1 if a barrier wait ran out.
+// FP64: xv (one column) receives each new vector in FP64 while V holds them
+// in fixed point, on systems whose w stays in shared memory; elsewhere V
+// holds FP64 columns and xv is not used.
+void arnoldi_step(const DevCsr& A, double* V, int64_t ld, int j, int k, double* xv, double* H,
                   int ldh, double* wn, double* red, int red_cap, unsigned* bar,
                   int* err, cudaStream_t st);
-// FP32 form: while j + 1 <= 161 and red holds prepass_red_doubles() the
+// FP32 form: while j + 1 <= 161 and red holds prepass_red_doubles(k) the
 // step takes two grid barriers (the MGS coefficients from the basis's Gram
 // matrix, whose rows it keeps in red across the steps of one pre-pass, so
 // the steps 0..k-1 of a pre-pass run in order on one red buffer).
 void arnoldi_step32(const DevCsr& A, float* V, int64_t ld, int j, double* H,
                     int ldh, double* wn, double* red, int red_cap, unsigned* bar,
                     int* err, cudaStream_t st);
-int64_t prepass_red_doubles();
+int64_t prepass_red_doubles(int k);
 // r = b - A x
 void residual(const DevCsr& A, const double* b, const double* x, double* r,
               cudaStream_t st);

@@ -52,11 +52,12 @@ Slots slots_for(int m, int k) {
 }
 
 // Partial sums of the streaming reductions (3 x reduction_blocks) and of
-// the cooperative pre-pass (the larger of the grouped step's 24 per SM and
-// the two-barrier step's partials plus its Gram rows).
-int red_doubles() {
+// the cooperative pre-pass of up to k steps (the largest of the grouped
+// step's 24 per SM, the two-barrier step's partials plus its Gram rows, and
+// the resident step's partials, exponents and exchange words).
+int red_doubles(int k) {
   return 3 * reduction_blocks() +
-         static_cast<int>(std::max<int64_t>(24 * device_sm_count(), prepass_red_doubles()));
+         static_cast<int>(std::max<int64_t>(24 * device_sm_count(), prepass_red_doubles(k)));
 }
 
 // Largest split-partials buffer over every block shape the solver uses
@@ -86,7 +87,7 @@ void ensure_workspace(sg_handle* h, int64_t n, int m, int k) {
   const int64_t part = max_part_size(n, m + 1, k);
   dev_alloc(&h->part, part);
   h->part_cap = part;
-  dev_alloc(&h->red, static_cast<size_t>(red_doubles()));
+  dev_alloc(&h->red, static_cast<size_t>(red_doubles(k)));
   Slots sl = slots_for(m, k);
   dev_alloc(&h->small, sl.total);
   h->small_cap = sl.total;
@@ -119,7 +120,7 @@ void ensure_workspace32(sg_handle* h, int64_t n, int m, int k) {
     const int64_t part = max_part_size(n, mm + 1, kk);
     dev_alloc(&h->part, part);
     h->part_cap = part;
-    dev_alloc(&h->red, static_cast<size_t>(red_doubles()));
+    dev_alloc(&h->red, static_cast<size_t>(red_doubles(kk)));
     Slots sl = slots_for(mm, kk);
     dev_alloc(&h->small, sl.total);
     h->small_cap = sl.total;
@@ -214,19 +215,19 @@ template <> struct Basis<float> {
 // the basis in V's columns (Sec. 3.4).  Returns the steps completed and
 // fills Hh ((k+1) x k, host, ld k+1).
 template <typename T>
-void step_kernel(const DevCsr& M, T* V, int64_t ld, int j, double* H, int ldh,
+void step_kernel(const DevCsr& M, T* V, int64_t ld, int j, int k, T* xv, double* H, int ldh,
                  double* wn, double* red, int red_cap, unsigned* bar, int* err,
                  cudaStream_t st);
 template <>
-void step_kernel<double>(const DevCsr& M, double* V, int64_t ld, int j, double* H,
-                         int ldh, double* wn, double* red, int red_cap, unsigned* bar,
-                         int* err, cudaStream_t st) {
-  arnoldi_step(M, V, ld, j, H, ldh, wn, red, red_cap, bar, err, st);
+void step_kernel<double>(const DevCsr& M, double* V, int64_t ld, int j, int k, double* xv,
+                         double* H, int ldh, double* wn, double* red, int red_cap,
+                         unsigned* bar, int* err, cudaStream_t st) {
+  arnoldi_step(M, V, ld, j, k, xv, H, ldh, wn, red, red_cap, bar, err, st);
 }
 template <>
-void step_kernel<float>(const DevCsr& M, float* V, int64_t ld, int j, double* H,
-                        int ldh, double* wn, double* red, int red_cap, unsigned* bar,
-                        int* err, cudaStream_t st) {
+void step_kernel<float>(const DevCsr& M, float* V, int64_t ld, int j, int, float*, double* H,
+                        int ldh, double* wn, double* red, int red_cap, unsigned* bar, int* err,
+                        cudaStream_t st) {
   arnoldi_step32(M, V, ld, j, H, ldh, wn, red, red_cap, bar, err, st);
 }
 
@@ -255,7 +256,7 @@ void enqueue_prepass(sg_handle* h, const DevCsr& M, const T* q, int k,
   SG_CUDA(cudaMemsetAsync(prepass_barrier(h), 0, 256, st));
   SG_CUDA(cudaMemcpyAsync(V, q, sizeof(T) * n, cudaMemcpyDeviceToDevice, st));
   for (int j = 0; j < k; ++j)
-    step_kernel<T>(M, V, ld, j, Hd, ldh, wn, h->red, red_doubles(),
+    step_kernel<T>(M, V, ld, j, k, B::Y(h), Hd, ldh, wn, h->red, red_doubles(h->ws_k),
                    prepass_barrier(h), prepass_error(h), st);
 }
 
