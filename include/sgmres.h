@@ -183,7 +183,7 @@ sg_status sg_gather(const int32_t* idx, int64_t count, const double* src, double
 
 /* Replace the values of the analysed matrix, keeping its pattern: val
  * has nnz entries (device pointer when on_device, else host).  The FP32
- * copy is refreshed and the transpose is rebuilt on the next adjoint
+ * copy is refreshed and the transpose takes them over on the next adjoint
  * call.  Errors: SG_ESTATE (no matrix), SG_EINVAL, SG_ECUDA. */
 sg_status sg_update_values(sg_handle* h, const double* val,
                            int32_t on_device);

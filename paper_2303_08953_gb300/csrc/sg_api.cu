@@ -59,6 +59,8 @@ void free_csr(sg::DevCsr& A) {
   if (A.sval32) cudaFree(A.sval32);
   if (A.sbase) cudaFree(A.sbase);
   if (A.soff) cudaFree(A.soff);
+  if (A.sperm) cudaFree(A.sperm);
+  if (A.src) cudaFree(A.src);
   A = sg::DevCsr();
 }
 
@@ -68,17 +70,16 @@ __global__ void f64_to_f32_kernel(int64_t n, const double* x, float* y) {
     y[i] = static_cast<float>(x[i]);
 }
 
-// FP32 copies of the values (CSR and, when present, SELL-32)
+// FP32 copies of the values (CSR and, when present, SELL-32), in the buffers
+// of an earlier call if there are any
 void make_val32(sg::DevCsr& A, cudaStream_t st) {
-  if (A.val32) cudaFree(A.val32);
-  A.val32 = nullptr;
-  if (A.sval32) cudaFree(A.sval32);
-  A.sval32 = nullptr;
-  SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&A.val32), sizeof(float) * std::max<int64_t>(A.nnz, 1)));
+  if (!A.val32)
+    SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&A.val32), sizeof(float) * std::max<int64_t>(A.nnz, 1)));
   f64_to_f32_kernel<<<sg::device_sm_count() * 8, 256, 0, st>>>(A.nnz, A.val, A.val32);
   SG_LAUNCH_CHECK();
   if (A.sptr) {
-    SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&A.sval32), sizeof(float) * A.sell_nnz));
+    if (!A.sval32)
+      SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&A.sval32), sizeof(float) * A.sell_nnz));
     f64_to_f32_kernel<<<sg::device_sm_count() * 8, 256, 0, st>>>(A.sell_nnz, A.sval, A.sval32);
     SG_LAUNCH_CHECK();
   }
@@ -176,28 +177,42 @@ void fill_result(const sg::SolveLog& L, sg_result* r) {
   r->fp64_iters = L.fp64_iters;
 }
 
-// A^T on the device (built on first use; values follow A's)
+// A^T on the device: its pattern, storage and the places of A's values in it
+// are laid out once per analysed pattern, the values follow A's.
 void ensure_transpose(sg_handle* h, cudaStream_t st) {
-  if (h->have_AT) return;
-  h->AT.n = h->A.n;
-  h->AT.nnz = h->A.nnz;
-  SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&h->AT.rowptr), sizeof(int32_t) * (h->A.n + 1)));
-  SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&h->AT.colind), sizeof(int32_t) * std::max<int64_t>(h->A.nnz, 1)));
-  SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&h->AT.val), sizeof(double) * std::max<int64_t>(h->A.nnz, 1)));
-  int32_t* counts = nullptr;
-  SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&counts), sizeof(int32_t) * (h->A.n + 1)));
-  try {
-    sg::csr_transpose(h->A, h->AT, counts, st);
-    SG_CUDA(cudaStreamSynchronize(st));
-  } catch (...) {
-    cudaFree(counts);
-    throw;
+  sg::DevCsr& T = h->AT;
+  if (h->have_AT && !h->at_stale) return;
+  if (!h->have_AT) {
+    const sg::DevCsr& A = h->A;
+    const size_t nz = static_cast<size_t>(std::max<int64_t>(A.nnz, 1));
+    int32_t* work = nullptr;
+    try {
+      T.n = A.n;
+      T.nnz = A.nnz;
+      SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&T.rowptr), sizeof(int32_t) * (A.n + 1)));
+      SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&T.colind), sizeof(int32_t) * nz));
+      SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&T.src), sizeof(int32_t) * nz));
+      SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&T.val), sizeof(double) * nz));
+      SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&work), sizeof(int32_t) * sg::transpose_work_ints(A)));
+      sg::csr_transpose(A, T, work, st);
+      sg::transpose_values(A, T, st);
+      SG_CUDA(cudaStreamSynchronize(st));
+      cudaFree(work);
+      work = nullptr;
+      T.mean_row = A.mean_row;
+      sg::build_sell(T, st);
+    } catch (...) {
+      if (work) cudaFree(work);
+      free_csr(T);
+      throw;
+    }
+    h->have_AT = true;
+  } else {
+    sg::transpose_values(h->A, T, st);
+    sg::sell_refill_values(T, st);
   }
-  cudaFree(counts);
-  h->AT.mean_row = h->A.mean_row;
-  sg::build_sell(h->AT, st);
-  if (h->A.val32) make_val32(h->AT, st);
-  h->have_AT = true;
+  if (T.val32 || h->A.val32) make_val32(T, st);
+  h->at_stale = false;
 }
 
 // the column-equilibrated matrix A D_c (its own value arrays only)
@@ -422,7 +437,7 @@ static sg_status analyze_impl(sg_handle* h, const sg_csr* A, int64_t ncols, bool
     free_equil(h);
     free_csr(h->A);
     free_csr(h->AT);
-    h->have_A = h->have_AT = false;
+    h->have_A = h->have_AT = h->at_stale = false;
     h->A = T;
     sg::DevCsr& D = h->A;
     D.mean_row = static_cast<double>(nnz) / static_cast<double>(n);
@@ -467,11 +482,7 @@ sg_status sg_update_values(sg_handle* h, const double* val, int32_t on_device) {
     if (h->A.nnz) copy_in(h->A.val, val, h->A.nnz, on_device != 0, st);
     sg::sell_refill_values(h->A, st);
     if (h->A.val32) make_val32(h->A, st);
-    if (h->have_AT) {  // values of the transpose are stale: rebuild lazily
-      h->drop_graphs();
-      free_csr(h->AT);
-      h->have_AT = false;
-    }
+    h->at_stale = true;  // the transpose takes them over on its next use
     SG_CUDA(cudaStreamSynchronize(st));
   });
 }

@@ -56,15 +56,22 @@ struct DevCsr {
   int32_t* scol = nullptr;
   double* sval = nullptr;
   float* sval32 = nullptr;
+  // Row order of the slices when rows were sorted by length within windows
+  // of kSellWindow rows (position -> row, -1 past the end); null: in order.
+  int32_t* sperm = nullptr;
   // The same columns as 16-bit offsets from each slice's smallest column
   // (0xFFFF marks padding), built when every slice spans fewer than 65535
   // columns: the SpMV then streams 10 bytes per stored entry instead of 12.
   int32_t* sbase = nullptr;  // nslices
   uint16_t* soff = nullptr;
+  // A transpose's entry p holds the value of entry src[p] of the original.
+  int32_t* src = nullptr;
 };
 
-// Build A's SELL-32 copy from its CSR arrays (kept when the padded size is
-// at most 1.2 nnz + 32 per slice and fits int32 offsets); frees any old one.
+// Build A's SELL-32 copy from its CSR arrays, with the rows in order or, when
+// that pads too much, sorted by length within windows of rows (kept when the
+// padded size is at most 1.2 nnz + 32 per slice and fits int32 offsets);
+// frees any old one.
 void build_sell(DevCsr& A, cudaStream_t st);
 // Copy A.val into the SELL value array after a value update.
 void sell_refill_values(const DevCsr& A, cudaStream_t st);
@@ -116,9 +123,12 @@ void residual(const DevCsr& A, const double* b, const double* x, double* r,
 // dval[k] = -lam[row(k)] * x[col(k)]
 void sampled_outer(const DevCsr& A, const double* lam, const double* x,
                    double* dval, cudaStream_t st);
-// CSR transpose (device to device), sorted columns.
-void csr_transpose(const DevCsr& A, DevCsr& T, int32_t* work_counts,
-                   cudaStream_t st);
+// CSR transpose (device to device), sorted columns: T's pattern and src
+// (arrays allocated by the caller).  work: transpose_work_ints(A) ints.
+int64_t transpose_work_ints(const DevCsr& A);
+void csr_transpose(const DevCsr& A, DevCsr& T, int32_t* work, cudaStream_t st);
+// T.val from A.val through src.
+void transpose_values(const DevCsr& A, const DevCsr& T, cudaStream_t st);
 
 // ------------------------------------------------------- vector kernels
 // Deterministic two-stage reductions: stage 1 writes `nred` per-block

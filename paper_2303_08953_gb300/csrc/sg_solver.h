@@ -12,6 +12,7 @@ struct sg_handle {
   sg::DevCsr A;      // the analysed matrix
   sg::DevCsr AT;     // its transpose (built on the first adjoint call)
   bool have_A = false, have_AT = false;
+  bool at_stale = false;   // A's values are newer than AT's
   bool rows_only = false;  // A is a row block (sg_analyze_rows): kernel-level calls only
   int64_t ncols = 0;       // columns of A (n for a square matrix)
   std::string err;
