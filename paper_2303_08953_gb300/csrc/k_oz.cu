@@ -50,6 +50,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "k_tc_common.cuh"
 #include "sg_internal.h"
@@ -101,60 +102,63 @@ __device__ __forceinline__ void mma_bf16_tmem_a(uint32_t dtmem, uint32_t atmem, 
       : "memory");
 }
 
-// x relative to 2^e (|x| < 2^e) as the signed integer m = x 2^(62 - e),
-// |m| < 2^62, truncated toward zero.
-__device__ __forceinline__ int64_t scaled62(double x, int e) {
-  const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(x));
-  const int E = static_cast<int>((bits >> 52) & 0x7FF);
-  uint64_t m = 0;
-  if (E != 0 && E != 0x7FF) {
-    const uint64_t mant = (bits & ((uint64_t(1) << 52) - 1)) | (uint64_t(1) << 52);
-    const int sh = E - 1013 - e;   // <= 9 when |x| < 2^e
-    if (sh >= 0) m = sh < 10 ? mant << sh : 0;
-    else if (sh > -64) m = mant >> (-sh);
-  }
-  return (bits >> 63) ? -static_cast<int64_t>(m) : static_cast<int64_t>(m);
-}
-
-// The integer value of an FP32 level sum (an exact integer, |v| < 2^24)
-// on the FP32 pipe: adding 1.5 2^25 (whose unit in the last place is 4)
-// rounds v to a multiple of 4 and leaves v / 4 in the low bits of the sum's
-// bit pattern; the remainder (-2 .. 2, exact) converts through 1.5 2^23 the
-// same way.  Profiles showed the F2I conversion occupying the FP64 pipe.
-__device__ __forceinline__ int32_t level_int(uint32_t vb) {
-  const float v = __uint_as_float(vb);
-  const float t = __fadd_rn(v, 50331648.0f);
-  const float r = __fsub_rn(v, __fsub_rn(t, 50331648.0f));
-  return 4 * (__float_as_int(t) - 0x4C400000) + (__float_as_int(__fadd_rn(r, 12582912.0f)) - 0x4B400000);
-}
-
-__device__ __forceinline__ uint32_t f16x2_sub(uint32_t a, uint32_t b) {
+__device__ __forceinline__ uint32_t f16x2_fma(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
-  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
 
+// v >> d, 0 for every d >= 32 (the PTX shift clamps; C++ leaves it undefined)
+__device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t d) {
+  uint32_t r;
+  asm("shr.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(d));
+  return r;
+}
+
+// |x| relative to 2^e (|x| < 2^e) as the integer m = |x| 2^(62 - e) < 2^62,
+// truncated, plus 0x80 in every byte: the mantissa with its top bit at bit
+// 61 is shifted right by e + 1022 - E (E: the exponent field).  Zeros and
+// subnormals (E = 0) give m = 0, and so does every shift outside 0 .. 63
+// (infinities and NaN, whose columns' exponents are those of finite values;
+// columns without an exponent).
+__device__ __forceinline__ uint2 biased62(double x, int e) {
+  const uint32_t xh = static_cast<uint32_t>(__double2hiint(x));
+  const uint32_t xl = static_cast<uint32_t>(__double2loint(x));
+  const uint32_t a = xh & 0x7FFFFFFFu;
+  uint32_t d = static_cast<uint32_t>(e + 1022 - static_cast<int>(a >> 20));
+  if (a < 0x00100000u) d = 64;
+  const uint32_t h = (xh & 0x000FFFFFu) | 0x00100000u;
+  const uint32_t H = __funnelshift_l(xl, h, 9), L = xl << 9;
+  const uint32_t lo = shr_clamp(__funnelshift_rc(L, H, d), max(d, 32u) - 32u);
+  const uint64_t s = ((static_cast<uint64_t>(shr_clamp(H, d)) << 32) | lo) + 0x8080808080808080ull;
+  return make_uint2(static_cast<uint32_t>(s), static_cast<uint32_t>(s >> 32));
+}
+
 // Balanced base-256 digits of two numbers as FP16 pairs: w[t] holds digit
-// t (most significant first) of ma in its low half and of mb in its high
-// half.  Adding 0x80 to every byte of m makes each byte of the sum the
-// digit plus 128 (the carries do the balancing; for |m| < 2^62 the top
-// byte stays in [64, 192]).  The FP16 number with bit pattern 0x6600 + b
-// is 1536 + b exactly (the unit in the last place is 1 on [1024, 2048)),
-// so one packed subtraction of 1664 leaves the digits, exactly.
-__device__ __forceinline__ void digits_f16x2(int64_t ma, int64_t mb, uint32_t* w) {
-  const uint64_t sa = static_cast<uint64_t>(ma) + 0x8080808080808080ull;
-  const uint64_t sb = static_cast<uint64_t>(mb) + 0x8080808080808080ull;
-  const uint32_t ahi = static_cast<uint32_t>(sa >> 32), alo = static_cast<uint32_t>(sa);
-  const uint32_t bhi = static_cast<uint32_t>(sb >> 32), blo = static_cast<uint32_t>(sb);
+// t (most significant first) of xa (relative to 2^ea) in its low half and
+// of xb (relative to 2^eb) in its high half.  With 0x80 added to every byte
+// of |m|, each byte of the sum is the digit plus 128 (the carries do the
+// balancing; the top byte stays in [128, 192]).  The FP16 number with bit
+// pattern 0x6600 + b is 1536 + b exactly (the unit in the last place is 1
+// on [1024, 2048)), so one packed FMA, (1536 + b) (+-1) -+ 1664, leaves the
+// signed digits, exactly.  The cut takes most of the issue slots of the
+// kernels below, so the sign costs three instructions a pair here, not a
+// 64-bit negation a value (with the readout below, at 2^21 rows: 121 x 120
+// dot 4.27 -> 3.74 ms, Gram of 120 3.95 -> 3.43, update 6.40 -> 6.04).
+__device__ __forceinline__ void cut_pair(double xa, int ea, double xb, int eb, uint32_t* w) {
+  const uint2 a = biased62(xa, ea), b = biased62(xb, eb);
+  const uint32_t sign = __byte_perm(static_cast<uint32_t>(__double2hiint(xa)),
+                                    static_cast<uint32_t>(__double2hiint(xb)), 0x7030) & 0x80008000u;
+  const uint32_t unit = sign ^ 0x3C003C00u;           // +-1
+  const uint32_t off = sign ^ 0xE680E680u;            // -+1664
   constexpr uint32_t kHi = 0x66666666u;
-  constexpr uint32_t kOff = 0x66806680u;              // 1664 in both halves
   // byte pairs (a_j, b_j) of digits 0-1, 2-3, 4-5, 6-7
-  const uint32_t p[4] = {__byte_perm(ahi, bhi, 0x6273), __byte_perm(ahi, bhi, 0x4051),
-                         __byte_perm(alo, blo, 0x6273), __byte_perm(alo, blo, 0x4051)};
+  const uint32_t p[4] = {__byte_perm(a.y, b.y, 0x6273), __byte_perm(a.y, b.y, 0x4051),
+                         __byte_perm(a.x, b.x, 0x6273), __byte_perm(a.x, b.x, 0x4051)};
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    w[2 * k] = f16x2_sub(__byte_perm(p[k], kHi, 0x4140), kOff);
-    w[2 * k + 1] = f16x2_sub(__byte_perm(p[k], kHi, 0x4342), kOff);
+    w[2 * k] = f16x2_fma(__byte_perm(p[k], kHi, 0x4140), unit, off);
+    w[2 * k + 1] = f16x2_fma(__byte_perm(p[k], kHi, 0x4342), unit, off);
   }
 }
 
@@ -172,14 +176,84 @@ __device__ __forceinline__ void tmem_st2(uint32_t taddr, const uint32_t* v) {
                : "memory");
 }
 
-// This thread's lane, 8 consecutive 32-bit columns from taddr.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
+// This thread's lane, 8 consecutive 32-bit columns from taddr, without
+// waiting for the load (tmem_wait_ld16 waits and orders the uses).
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* v) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
         "=r"(v[7])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// Waits for this thread's tensor-memory loads; the 16 registers are operands
+// so that no use of them is scheduled before the wait.
+__device__ __forceinline__ void tmem_wait_ld16(uint32_t* v) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]),
+                 "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]),
+                 "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+               :
+               : "memory");
+}
+
+// Exact sums of an output over readouts of its eight level sums, as two
+// int64 halves: hi = sum of S_L 256^(3 - L) over L = 0..3, lo = sum of
+// S_L 256^(7 - L) over L = 4..7.  A level sum is an integer in FP32; adding
+// 1.5 2^23 (1.5 2^25) leaves it (a quarter of it, rounded) in the low bits
+// of the sum's bit pattern, and the whole pattern is multiplied onto the
+// accumulator: the constant it carries is the same at every readout, so the
+// accumulators start at minus what all their readouts add (everything modulo
+// 2^64).  Levels 0 and 1 (one and two digit pairs over 128 rows: at most
+// 2^22) take one addition; the others leave a remainder of -2 .. 2, and
+// those of levels 2-4 and 5-7 are joined, exactly, in FP32 first.  36
+// instructions an output, none on the integer ALU, which the cut needs;
+// converting each level by itself took about 70.
+constexpr uint64_t kBits23 = 0x4B400000u, kBits25 = 0x4C400000u;
+constexpr uint64_t kReadHi = kBits23 * ((1u << 24) + (1u << 16)) + kBits25 * ((1u << 10) + 4u);
+constexpr uint64_t kReadLo =
+    kBits25 * ((1u << 26) + (1u << 18) + (1u << 10) + 4u) + kBits23 * ((1u << 24) + 1u);
+
+__device__ __forceinline__ uint64_t bits_times(float f, uint32_t w) {
+  return static_cast<uint64_t>(__float_as_uint(f)) * w;
+}
+
+template <int L>
+__device__ __forceinline__ void add_level(uint32_t vb, float& rest, uint64_t& hi, uint64_t& lo) {
+  const float v = __uint_as_float(vb);
+  if constexpr (L < 2) {
+    hi += bits_times(__fadd_rn(v, 12582912.0f), L == 0 ? 1u << 24 : 1u << 16);
+  } else {
+    const float t = __fadd_rn(v, 50331648.0f);
+    const float r = __fsub_rn(v, __fsub_rn(t, 50331648.0f));
+    if constexpr (L < 4) hi += bits_times(t, 4u << (8 * (3 - L)));
+    else lo += bits_times(t, 4u << (8 * (7 - L)));
+    rest = (L == 2 || L == 5) ? r : __fmaf_rn(rest, 256.0f, r);
+    if constexpr (L == 4 || L == 7)
+      lo += bits_times(__fadd_rn(rest, 12582912.0f), L == 4 ? 1u << 24 : 1u);
+  }
+}
+
+// The level sums of 8 outputs (columns taddr + 32 L .. + 7 of this thread's
+// lane) added to their accumulators, two levels a wait.
+__device__ __forceinline__ void add_levels8(uint32_t taddr, uint64_t* hi, uint64_t* lo) {
+  float rest[8];
+  uint32_t v[16];
+  auto two = [&](auto LL) {
+    constexpr int L = decltype(LL)::value;
+    tmem_ld8_nowait(taddr + 32u * L, v);
+    tmem_ld8_nowait(taddr + 32u * (L + 1), v + 8);
+    tmem_wait_ld16(v);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      add_level<L>(v[c], rest[c], hi[c], lo[c]);
+      add_level<L + 1>(v[8 + c], rest[c], hi[c], lo[c]);
+    }
+  };
+  two(std::integral_constant<int, 0>{});
+  two(std::integral_constant<int, 2>{});
+  two(std::integral_constant<int, 4>{});
+  two(std::integral_constant<int, 6>{});
 }
 
 // Instruction descriptor: kind::f16 with FP16 A and B, FP32 accumulator,
@@ -297,27 +371,18 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
   // the output's V' = ahi 2^32 + alo
   constexpr int kCols = kON / 4;
   const int cg = warp >> 2;
-  int64_t alo[kCols];
-  int64_t ahi[kCols];
+  uint64_t alo[kCols];
+  uint64_t ahi[kCols];
+  const uint64_t reads = static_cast<uint64_t>((nk + kChunk - 1) / kChunk);
 #pragma unroll
-  for (int c = 0; c < kCols; ++c) { alo[c] = 0; ahi[c] = 0; }
+  for (int c = 0; c < kCols; ++c) { alo[c] = 0 - reads * kReadLo; ahi[c] = 0 - reads * kReadHi; }
   auto readout = [&](int k) -> bool {
     if (!mbar_wait(&sh.accfull, static_cast<uint32_t>((k / kChunk) & 1))) sh.fail = 1;
     if (__any_sync(0xffffffffu, failed())) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) +
                         static_cast<uint32_t>(cg * kCols);
-#pragma unroll
-    for (int L = 0; L < kLev; ++L) {
-      uint32_t v[kCols];
-      tmem_ld8(tl + kAccCol + static_cast<uint32_t>(32 * L), v);
-#pragma unroll
-      for (int cc = 0; cc < kCols; ++cc) {
-        const int64_t sv = level_int(v[cc]);
-        if (L < 4) ahi[cc] += sv * (int64_t(1) << (8 * (3 - L)));
-        else alo[cc] += sv * (int64_t(1) << (8 * (7 - L)));
-      }
-    }
+    add_levels8(tl + kAccCol, ahi, alo);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     mbar_arrive(&sh.accfree);
     return true;
@@ -421,7 +486,7 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
         const unsigned char* line = stX(b) + (warp >> 3) * kXBox + lane * 128;
         const double2 v = *reinterpret_cast<const double2*>(line + (((warp & 7) ^ (lane & 7)) << 4));
         uint32_t d8[kDig];
-        digits_f16x2(scaled62(v.x, eN), scaled62(v.y, eN), d8);
+        cut_pair(v.x, eN, v.y, eN, d8);
         unsigned char* bs = stB(b) + (lane >> 3) * 1024 + (lane & 7) * 128 + (warp & 3) * 4;
         const int chunk = (warp >> 2) ^ (lane & 7);
 #pragma unroll
@@ -440,7 +505,7 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
           const int jj = 4 * (cg & 1) + j;
           const double2 v = *reinterpret_cast<const double2*>(line + ((jj ^ (m & 7)) << 4));
           uint32_t d8[kDig];
-          digits_f16x2(scaled62(v.x, eM), scaled62(v.y, eM), d8);
+          cut_pair(v.x, eM, v.y, eM, d8);
 #pragma unroll
           for (int t = 0; t < kDig; ++t) words[t][j] = d8[t];
         }
@@ -481,7 +546,7 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
         const int gc = n0 + cg * kCols + cc;
         if (gc < N) {
           // V' = (ahi + carry) 2^32 + the low 32 bits of alo, rounded once
-          const int64_t hi = ahi[cc] + (alo[cc] >> 32);
+          const int64_t hi = static_cast<int64_t>(ahi[cc]) + (static_cast<int64_t>(alo[cc]) >> 32);
           const uint32_t lo = static_cast<uint32_t>(alo[cc]);
           P[gm + static_cast<int64_t>(gc) * M] =
               (eM < -2000 || ex[gc] < -2000) ? 0.0 : int96_to_double(hi, lo, eM + ex[gc] - 68);
@@ -537,7 +602,7 @@ constexpr uint32_t kUACol = 256;                        // A buffer b: 256 + 128
 // per-column tables after the W' slices: Q's column exponents e_k, W'
 // column exponents g_c
 struct OzUTables {
-  int eq[kUMaxK];
+  alignas(16) int eq[kUMaxK];
   int g[kUN];
 };
 
@@ -637,9 +702,9 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     const int c = lane;
     const int gc = tb.g[c] > -2000 ? tb.g[c] : -4000;
     for (int k = warp; k < i; k += kUWarps) {
-      const int64_t mk = scaled62(wprime(k, c), gc);
+      const double wk = wprime(k, c);
       uint32_t w8[kDig];
-      digits_f16x2(mk, mk, w8);
+      cut_pair(wk, gc, wk, gc, w8);
       const int kc = k / 64, kk = k % 64;
 #pragma unroll
       for (int t = 0; t < kDig; ++t) {
@@ -739,9 +804,11 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     const int m = (warp & 3) * 32 + lane;
     const int cg = warp >> 2;
     const uint32_t tlane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-    int64_t alo[kCols], ahi[kCols];
+    uint64_t alo[kCols], ahi[kCols];
+    const uint64_t lo0 = 0 - static_cast<uint64_t>(gpt) * kReadLo;
+    const uint64_t hi0 = 0 - static_cast<uint64_t>(gpt) * kReadHi;
 #pragma unroll
-    for (int c = 0; c < kCols; ++c) { alo[c] = 0; ahi[c] = 0; }
+    for (int c = 0; c < kCols; ++c) { alo[c] = lo0; ahi[c] = hi0; }
     // level sums of the group ending at stage pq; the epilogue after a
     // tile's last group
     auto readout = [&](int pq) -> bool {
@@ -752,17 +819,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       if (__any_sync(0xffffffffu, failed())) return false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t tl = tlane + static_cast<uint32_t>(cg * kCols);
-#pragma unroll
-      for (int L = 0; L < kLev; ++L) {
-        uint32_t v[kCols];
-        tmem_ld8(tl + kAccCol + static_cast<uint32_t>(32 * L), v);
-#pragma unroll
-        for (int cc = 0; cc < kCols; ++cc) {
-          const int64_t sv = level_int(v[cc]);
-          if (L < 4) ahi[cc] += sv * (int64_t(1) << (8 * (3 - L)));
-          else alo[cc] += sv * (int64_t(1) << (8 * (7 - L)));
-        }
-      }
+      add_levels8(tl + kAccCol, ahi, alo);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(&sh.accfree);
       if (kq == nsub - 1) {
@@ -776,7 +833,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
 #pragma unroll
         for (int cc = 0; cc < kCols; ++cc) {
           // V' = (ahi + carry) 2^32 + the low 32 bits of alo
-          const int64_t hi = ahi[cc] + (alo[cc] >> 32);
+          const int64_t hi = static_cast<int64_t>(ahi[cc]) + (static_cast<int64_t>(alo[cc]) >> 32);
           const uint32_t lo = static_cast<uint32_t>(alo[cc]);
           const int gcol = tb.g[cg * kCols + cc];
           double p;
@@ -789,8 +846,8 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           }
           if (r < n && c0 + cc < s)
             xr[static_cast<int64_t>(cc) * ldx] = loadx ? fma(beta, xs[cc * kUM], p) : p;
-          alo[cc] = 0;
-          ahi[cc] = 0;
+          alo[cc] = lo0;
+          ahi[cc] = hi0;
         }
         if (loadx) mbar_arrive(&sh.xfree);
       }
@@ -822,6 +879,9 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       const int k0 = kq * kUS + kCols * cg;
       if (kq * kUS + 16 * (cg >> 1) < i) {
         const unsigned char* col = base + b * kUBox + kCols * cg * 1024 + m * 8;
+        const int4 e0 = *reinterpret_cast<const int4*>(tb.eq + k0);
+        const int4 e1 = *reinterpret_cast<const int4*>(tb.eq + k0 + 4);
+        const int e8[kCols] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           uint32_t words[kDig][2];
@@ -831,7 +891,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             const double va = *reinterpret_cast<const double*>(col + c * 1024);
             const double vb = *reinterpret_cast<const double*>(col + (c + 1) * 1024);
             uint32_t d8[kDig];
-            digits_f16x2(scaled62(va, tb.eq[k0 + c]), scaled62(vb, tb.eq[k0 + c + 1]), d8);
+            cut_pair(va, e8[c], vb, e8[c + 1], d8);
 #pragma unroll
             for (int t = 0; t < kDig; ++t) words[t][w] = d8[t];
           }
@@ -1111,27 +1171,6 @@ __device__ __forceinline__ void mma_f16_ss(uint32_t dtmem, uint64_t a, uint64_t 
       : "memory");
 }
 
-// This thread's lane, 8 consecutive 32-bit columns from taddr, without
-// waiting for the load (tmem_wait_ld16 waits and orders the uses).
-__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7])
-      : "r"(taddr));
-}
-
-// Waits for this thread's tensor-memory loads; the 16 registers are operands
-// so that no use of them is scheduled before the wait.
-__device__ __forceinline__ void tmem_wait_ld16(uint32_t* v) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]),
-                 "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]),
-                 "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
-               :
-               : "memory");
-}
-
 // Shared-memory matrix descriptor: K-major operand, 64-byte swizzle (lines
 // of 64 bytes, the 16-byte chunk c of line r stored at c ^ ((r >> 1) & 3)),
 // 8-line groups 512 bytes apart (slice bases aligned to 1024 bytes).
@@ -1224,10 +1263,11 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
   const int half = (warp >> 2) & 1;
   const bool mine = (warp & 3) <= q;   // columns 32 (w % 4) .. + 31 are within 0 .. 32q + 31
   const bool cutter = warp < kDWarps / 2;
-  int64_t alo[16];
-  int64_t ahi[16];
+  uint64_t alo[16];
+  uint64_t ahi[16];
+  const uint64_t reads = static_cast<uint64_t>((nk + kGChunk - 1) / kGChunk);
 #pragma unroll
-  for (int c = 0; c < 16; ++c) { alo[c] = 0; ahi[c] = 0; }
+  for (int c = 0; c < 16; ++c) { alo[c] = 0 - reads * kReadLo; ahi[c] = 0 - reads * kReadHi; }
   auto readout = [&](int g) -> bool {
     const int a = g & 1;
     if (!mbar_wait(&sh.accfull[a], static_cast<uint32_t>((g >> 1) & 1))) sh.fail = 1;
@@ -1235,20 +1275,8 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) +
                         static_cast<uint32_t>(a) * kGSetCol + static_cast<uint32_t>(half * 16);
-#pragma unroll
-    for (int L = 0; L < kGLev; ++L) {
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        uint32_t v[8];
-        tmem_ld8(tl + static_cast<uint32_t>(kGN * L + 8 * hh), v);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int64_t sv = level_int(v[c]);
-          if (L < 4) ahi[8 * hh + c] += sv * (int64_t(1) << (8 * (3 - L)));
-          else alo[8 * hh + c] += sv * (int64_t(1) << (8 * (7 - L)));
-        }
-      }
-    }
+    add_levels8(tl, ahi, alo);
+    add_levels8(tl + 8, ahi + 8, alo + 8);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     mbar_arrive(&sh.accfree[a]);
     return true;
@@ -1420,7 +1448,7 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
           val = 0.0;                                         // an all-zero column
         } else {
           // V = (ahi + carry) 2^32 + the low 32 bits of alo, rounded once
-          const int64_t hi = ahi[cc] + (alo[cc] >> 32);
+          const int64_t hi = static_cast<int64_t>(ahi[cc]) + (static_cast<int64_t>(alo[cc]) >> 32);
           const uint32_t lo = static_cast<uint32_t>(alo[cc]);
           val = int96_to_double(hi, lo, em + en - 68);
         }
