@@ -40,6 +40,10 @@
 //     0 .. 7 (36 MMAs of N = 32 would issue the same tensor work);
 //     every four stages, one stage late, they read the level sums, eight
 //     output columns each.
+// A stage takes about 3,300 cycles: 2,200 the cut, 700 (a quarter of a
+// readout) the level sums, 400 waits; the MMAs' 1,800 overlap the cut.  At
+// 2^21 rows the 121 x 120 dot takes 3.61 ms with the exponents (4.27 before
+// the cut and the readout were shortened), the Gram of 120 3.30 ms (3.95).
 // Every wait is bounded: on timeout the kernel records an error, drains
 // its own copies, frees its tensor memory and returns.
 #include <cuda.h>
@@ -134,23 +138,58 @@ __device__ __forceinline__ uint2 biased62(double x, int e) {
   return make_uint2(static_cast<uint32_t>(s), static_cast<uint32_t>(s >> 32));
 }
 
+// The same for |x| in [2^(e - 32), 2^e), where the shift is 1 .. 31 (the
+// mantissa's top bit at bit 62 first), from the column's word
+// w = near_word(e): E + w is minus the shift modulo 32.  It needs neither the
+// clamps nor the test for E = 0 of the general form above.  (Written as
+// multiply-adds, which the compiler turns into shifts and additions where
+// they are cheaper; with factors it cannot see, all of it on the FMA pipe,
+// the kernels were 3 % slower.)
+__device__ __forceinline__ uint2 biased62_near(uint32_t xh, uint32_t xl, uint32_t w, uint32_t one) {
+  const uint32_t h = ((xh << 10) & 0x3FFFFFFFu) | 0x40000000u;
+  uint64_t m, sh, r;
+  asm("mad.wide.u32 %0, %1, 1024, %2;" : "=l"(m) : "r"(xl), "l"(static_cast<uint64_t>(h) << 32));
+  asm("mad.wide.u32 %0, %1, 4096, %2;" : "=l"(sh) : "r"(xh), "l"(static_cast<uint64_t>(w) << 32));
+  const uint32_t H = static_cast<uint32_t>(m >> 32), c = static_cast<uint32_t>(sh >> 32);
+  const uint32_t lo = __funnelshift_l(static_cast<uint32_t>(m), H, c);
+  const uint32_t hi = __funnelshift_l(H, 0u, c);
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(lo), "r"(one), "l"(0x8080808080808080ull));
+  return make_uint2(static_cast<uint32_t>(r), hi * one + static_cast<uint32_t>(r >> 32));
+}
+
+// A column's word for biased62_near: the smallest exponent field it takes,
+// E0 = max(e - 31 + 1023, 1), in the top 11 bits, and -(e + 1023) modulo 32
+// in the low 5.  w - 2 xh (modulo 2^32) exceeds kNearMin only for
+// E0 <= E < E0 + 31 (and for all of these but up to 2^-15 of the lowest and
+// of the highest binade, which the general form then takes), so the smallest
+// one tells whether all of a thread's values may go this way: not zeros,
+// subnormals, infinities, NaN or values far below their column's largest.
+// For a column without an exponent (all zero, or outside the matrix; its
+// digits are never used) zeros pass.
+constexpr uint32_t kNearMin = 0xFFFFFFFFu - (31u << 21) + 32u;
+
+__device__ __forceinline__ uint32_t near_word(int e) {
+  if (e < -2000) return 0xFFFFFFE0u;
+  return (static_cast<uint32_t>(max(e + 992, 1)) << 21) | (static_cast<uint32_t>(-(e + 1023)) & 31u);
+}
+
+__device__ __forceinline__ uint32_t near_test(double x, uint32_t w) {
+  return w - 2u * static_cast<uint32_t>(__double2hiint(x));
+}
+
 // Balanced base-256 digits of two numbers as FP16 pairs: w[t] holds digit
-// t (most significant first) of xa (relative to 2^ea) in its low half and
-// of xb (relative to 2^eb) in its high half.  With 0x80 added to every byte
-// of |m|, each byte of the sum is the digit plus 128 (the carries do the
-// balancing; the top byte stays in [128, 192]).  The FP16 number with bit
-// pattern 0x6600 + b is 1536 + b exactly (the unit in the last place is 1
-// on [1024, 2048)), so one packed FMA, (1536 + b) (+-1) -+ 1664, leaves the
-// signed digits, exactly.  The cut takes most of the issue slots of the
-// kernels below, so the sign costs three instructions a pair here, not a
-// 64-bit negation a value (with the readout below, at 2^21 rows: 121 x 120
-// dot 4.27 -> 3.74 ms, Gram of 120 3.95 -> 3.43, update 6.40 -> 6.04).
-__device__ __forceinline__ void cut_pair(double xa, int ea, double xb, int eb, uint32_t* w) {
-  const uint2 a = biased62(xa, ea), b = biased62(xb, eb);
+// t (most significant first) of xa in its low half and of xb in its high
+// half.  With 0x80 added to every byte of |m|, each byte of the sum is the
+// digit plus 128 (the carries do the balancing; the top byte stays in
+// [128, 192]).  The FP16 number with bit pattern 0x6600 + b is 1536 + b
+// exactly (the unit in the last place is 1 on [1024, 2048)), so one packed
+// FMA, (1536 + b) (+-1) -+ 1664, leaves the signed digits, exactly: the sign
+// costs three instructions a pair, not a 64-bit negation a value.
+__device__ __forceinline__ void digits_f16x2(uint2 a, uint2 b, double xa, double xb, uint32_t* w) {
   const uint32_t sign = __byte_perm(static_cast<uint32_t>(__double2hiint(xa)),
-                                    static_cast<uint32_t>(__double2hiint(xb)), 0x7030) & 0x80008000u;
-  const uint32_t unit = sign ^ 0x3C003C00u;           // +-1
-  const uint32_t off = sign ^ 0xE680E680u;            // -+1664
+                                    static_cast<uint32_t>(__double2hiint(xb)), 0x7030);
+  const uint32_t unit = (sign & 0x80008000u) ^ 0x3C003C00u;   // +-1
+  const uint32_t off = (sign & 0x80008000u) ^ 0xE680E680u;    // -+1664
   constexpr uint32_t kHi = 0x66666666u;
   // byte pairs (a_j, b_j) of digits 0-1, 2-3, 4-5, 6-7
   const uint32_t p[4] = {__byte_perm(a.y, b.y, 0x6273), __byte_perm(a.y, b.y, 0x4051),
@@ -160,6 +199,20 @@ __device__ __forceinline__ void cut_pair(double xa, int ea, double xb, int eb, u
     w[2 * k] = f16x2_fma(__byte_perm(p[k], kHi, 0x4140), unit, off);
     w[2 * k + 1] = f16x2_fma(__byte_perm(p[k], kHi, 0x4342), unit, off);
   }
+}
+
+// xa relative to 2^ea and xb relative to 2^eb, any values
+__device__ __forceinline__ void cut_pair(double xa, int ea, double xb, int eb, uint32_t* w) {
+  digits_f16x2(biased62(xa, ea), biased62(xb, eb), xa, xb, w);
+}
+
+// both near their columns' largest (words wa, wb)
+__device__ __forceinline__ void cut_pair_near(double xa, uint32_t wa, double xb, uint32_t wb,
+                                              uint32_t one, uint32_t* w) {
+  digits_f16x2(biased62_near(static_cast<uint32_t>(__double2hiint(xa)),
+                             static_cast<uint32_t>(__double2loint(xa)), wa, one),
+               biased62_near(static_cast<uint32_t>(__double2hiint(xb)),
+                             static_cast<uint32_t>(__double2loint(xb)), wb, one), xa, xb, w);
 }
 
 // This thread's lane, 4 consecutive 32-bit columns from taddr.
@@ -462,6 +515,14 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
     const int eM = (m0 + m < M) ? eq[m0 + m] : -4000;
     const int eN = (n0 + lane < N) ? ex[n0 + lane] : -4000;
     const uint32_t tlane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    const uint32_t wM = near_word(eM), wN = near_word(eN);
+    const uint32_t one = blockDim.z;   // 1
+    // offsets of this thread's lines and chunks in the Q and X boxes (128-byte
+    // swizzle) and of its digits in a B slice
+    const int qoff = (cg >> 1) * kQBox + m * 128 + (((4 * (cg & 1)) ^ (m & 7)) << 4);
+    const int xoff = (warp >> 3) * kXBox + lane * 128 + (((warp & 7) ^ (lane & 7)) << 4);
+    const int boff = (lane >> 3) * 1024 + (lane & 7) * 128 + (warp & 3) * 4 +
+                     (((warp >> 2) ^ (lane & 7)) << 4);
     int pend = -1;
     bool stop = false;
     for (int k = 0; k < nk; ++k) {
@@ -480,39 +541,43 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      {
-        // B: rows 2w, 2w + 1 of X column `lane`, one FP16 pair per digit at
-        // K offset 2w of the column's 128-byte swizzled row
-        const unsigned char* line = stX(b) + (warp >> 3) * kXBox + lane * 128;
-        const double2 v = *reinterpret_cast<const double2*>(line + (((warp & 7) ^ (lane & 7)) << 4));
-        uint32_t d8[kDig];
-        cut_pair(v.x, eN, v.y, eN, d8);
-        unsigned char* bs = stB(b) + (lane >> 3) * 1024 + (lane & 7) * 128 + (warp & 3) * 4;
-        const int chunk = (warp >> 2) ^ (lane & 7);
+      // A (Q): column m's rows 8 cg .. + 7: box cg / 2, chunks
+      // 4 (cg % 2) + j (rows 2j, 2j + 1 of the box) -> tensor-memory column
+      // 4 cg + j of each digit slice of buffer b;
+      // B (X): rows 2w, 2w + 1 of X column `lane`, one FP16 pair per digit at
+      // K offset 2w of the column's 128-byte swizzled row
+      double2 va[4];
+      uint32_t ta = 0xFFFFFFFFu;
 #pragma unroll
-        for (int t = 0; t < kDig; ++t)
-          *reinterpret_cast<uint32_t*>(bs + t * kBSlice + (chunk << 4)) = d8[t];
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      for (int j = 0; j < 4; ++j) {
+        va[j] = *reinterpret_cast<const double2*>(stQ(b) + (qoff ^ (j << 4)));
+        ta = min(ta, min(near_test(va[j].x, wM), near_test(va[j].y, wM)));
       }
-      {
-        // A: column m's rows 8 cg .. + 7: box cg / 2, chunks 4 (cg % 2) + j
-        // (rows 2j, 2j + 1 of the box) -> tensor-memory column 4 cg + j of
-        // each digit slice of buffer b
-        const unsigned char* line = stQ(b) + (cg >> 1) * kQBox + m * 128;
+      const double2 vb = *reinterpret_cast<const double2*>(stX(b) + xoff);
+      ta = min(ta, min(near_test(vb.x, wN), near_test(vb.y, wN)));
+      auto cut = [&](auto near) {
+        constexpr bool kNear = decltype(near)::value;
+        uint32_t d8[kDig];
+        if (kNear) cut_pair_near(vb.x, wN, vb.y, wN, one, d8);
+        else cut_pair(vb.x, eN, vb.y, eN, d8);
+        unsigned char* bs = stB(b) + boff;
+#pragma unroll
+        for (int t = 0; t < kDig; ++t) *reinterpret_cast<uint32_t*>(bs + t * kBSlice) = d8[t];
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         uint32_t words[kDig][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int jj = 4 * (cg & 1) + j;
-          const double2 v = *reinterpret_cast<const double2*>(line + ((jj ^ (m & 7)) << 4));
-          uint32_t d8[kDig];
-          cut_pair(v.x, eM, v.y, eM, d8);
+          if (kNear) cut_pair_near(va[j].x, wM, va[j].y, wM, one, d8);
+          else cut_pair(va[j].x, eM, va[j].y, eM, d8);
 #pragma unroll
           for (int t = 0; t < kDig; ++t) words[t][j] = d8[t];
         }
 #pragma unroll
         for (int t = 0; t < kDig; ++t)
           tmem_st4(tlane + kDACol + static_cast<uint32_t>(128 * b + 16 * t + 4 * cg), words[t]);
-      }
+      };
+      if (__all_sync(0xffffffffu, ta > kNearMin)) cut(std::true_type{});
+      else cut(std::false_type{});
       mbar_arrive(&sh.qfree[b]);
       tmem_st_wait();
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -590,7 +655,14 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
 //     end of a tile, one stage late so that the split of the next stage
 //     overlaps the last MMAs; the epilogue writes beta X + alpha V 2^(g_c-68)
 //     from the prefetched X box.
-// K steps that lie wholly beyond column i are not issued.
+// K steps that lie wholly beyond column i are not issued, and with W upper
+// triangular a column tile stops at Q's columns 0 .. 32 ct + 31.
+// What bounds it: the cut (about 2,200 of the 3,300 cycles of a stage; the
+// MMAs, eight of N = 256 .. 32 each 16 columns, take 1,800 and overlap it),
+// then the readout and the epilogue, which the MMAs wait for.  At 2^21 rows:
+// 121 x 120 4.69 ms (6.40 with the general cut, a level at a time and the
+// product with alpha on the FP64 pipe), the triangular product of 120
+// 3.96 ms (6.33; 5.30 of it from leaving out W's lower triangle).
 constexpr int kUM = 128;
 constexpr int kUN = 32;
 constexpr int kUS = 32;                                 // columns of Q per stage
@@ -599,10 +671,10 @@ constexpr int kUBox = kUM * kUS * 8;                    // 32 KB: a Q stage or t
 constexpr int kUBChunk = kDig * kBSlice;                // 32 KB per 64 columns of Q
 constexpr uint32_t kUACol = 256;                        // A buffer b: 256 + 128 b
 
-// per-column tables after the W' slices: Q's column exponents e_k, W'
-// column exponents g_c
+// per-column tables after the W' slices: the words of Q's column exponents
+// e_k, W' column exponents g_c
 struct OzUTables {
-  alignas(16) int eq[kUMaxK];
+  alignas(16) uint32_t w[kUMaxK];
   int g[kUN];
 };
 
@@ -620,7 +692,25 @@ int oz_update_smem(int i) {
          static_cast<int>(sizeof(OzUShared)) + 1024;
 }
 
-// grid: (tiles of 32 X columns, row groups); row tiles g, g + G, ...
+// The CTAs of column tile ct are first(ct) .. first(ct + 1) - 1 of the grid's
+// P >= ntc: at least one each, the rest in proportion to the tile's work, a
+// fixed part (readout, epilogue) and its 16-column steps of Q.  With W upper
+// triangular, column tile ct needs only Q's columns 0 .. 32 ct + 31.
+constexpr int kUTileW = 6;                              // fixed part, in steps
+
+__host__ __device__ inline int oz_update_first(int ct, int ntc, int i, int upper, int P) {
+  int64_t before = 0, all = 0;
+  for (int c = 0; c < ntc; ++c) {
+    const int k = upper && i > (c + 1) * kUN ? (c + 1) * kUN : i;
+    const int w = kUTileW + (k + 15) / 16;
+    if (c < ct) before += w;
+    all += w;
+  }
+  return ct + static_cast<int>((P - ntc) * before / all);
+}
+
+// grid: CTAs of every column tile in turn; the g-th of a tile's G takes row
+// tiles g, g + G, ...
 __global__ void __launch_bounds__(kUThreads, 1)
 oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapX,
                  int64_t n, int i, int s, const double* __restrict__ W, int ldw,
@@ -632,10 +722,20 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
-  const int n0 = blockIdx.x * kUN;
+  // this CTA's column tile, its place among the tile's CTAs and their number
+  const int ntc = (s + kUN - 1) / kUN;
+  int ct = 0, first = 0, next = oz_update_first(1, ntc, i, upper, gridDim.x);
+  while (static_cast<int>(blockIdx.x) >= next) {
+    ++ct;
+    first = next;
+    next = oz_update_first(ct + 1, ntc, i, upper, gridDim.x);
+  }
+  const int g0 = static_cast<int>(blockIdx.x) - first;
+  const int G = next - first;
+  const int n0 = ct * kUN;
+  if (upper && i > n0 + kUN) i = n0 + kUN;       // W is zero below
   const int64_t ntiles = (n + kUM - 1) / kUM;
-  const int G = gridDim.y;
-  const int my_tiles = static_cast<int>((ntiles - blockIdx.y + G - 1) / G);
+  const int my_tiles = g0 < ntiles ? static_cast<int>((ntiles - g0 + G - 1) / G) : 0;
   const int nsub = (i + kUS - 1) / kUS;          // stages per row tile
   const int nkc = (i + 63) / 64;                 // groups of W' slices
   const int gpt = (nsub + 3) / 4;                // level readouts per row tile
@@ -646,10 +746,13 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   OzUShared& sh = *reinterpret_cast<OzUShared*>(bsl + nkc * kUBChunk + sizeof(OzUTables));
   auto failed = [&]() { return *reinterpret_cast<volatile int*>(&sh.fail) != 0; };
   auto group_end = [&](int kq) { return (kq & 3) == 3 || kq == nsub - 1; };
-  // alpha = +-2^(ka - 1) folds into the exponent and the sign of the sums
-  int ka = 0;
-  const double fa = frexp(alpha, &ka);
-  const bool apow2 = fabs(fa) == 0.5;
+  // alpha = +-2^ka folds into the exponent and the sign of the sums (all of
+  // it in integers: a product and a sign on the FP64 pipe for every output
+  // kept that pipe busy longer than the one addition the outputs need)
+  const uint64_t abits = static_cast<uint64_t>(__double_as_longlong(alpha));
+  const uint64_t asign = abits & (uint64_t(1) << 63);
+  const int ka = static_cast<int>((abits >> 52) & 0x7FF) - 1023;
+  const bool apow2 = (abits << 12) == 0 && ka > -1023 && ka < 1024;
 
   if (tid == 0) {
     for (int b = 0; b < 2; ++b) {
@@ -676,7 +779,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   // W' = W 2^(e_k) (zero below the diagonal when `upper`) cut into digits
   // relative to its column exponents g_c: B slices of every 64 columns of Q
   if (warp < kUWarps) {
-    for (int k = tid; k < kUMaxK; k += kUSplit) tb.eq[k] = k < i ? eq[k] : -4000;
+    for (int k = tid; k < kUMaxK; k += kUSplit) tb.w[k] = near_word(k < i ? eq[k] : -4000);
     if (tid < kUN) tb.g[tid] = -2147483647;
     uint4* z = reinterpret_cast<uint4*>(bsl);
     for (int e = tid; e < nkc * kUBChunk / 16; e += kUSplit) z[e] = make_uint4(0, 0, 0, 0);
@@ -684,8 +787,8 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   __syncthreads();
   auto wprime = [&](int k, int c) -> double {
     const int gc = n0 + c;
-    if (k >= i || gc >= s || (upper && k > gc) || tb.eq[k] < -2000) return 0.0;
-    return ldexp(W[k + static_cast<int64_t>(gc) * ldw], tb.eq[k]);
+    if (k >= i || gc >= s || (upper && k > gc) || eq[k] < -2000) return 0.0;
+    return ldexp(W[k + static_cast<int64_t>(gc) * ldw], eq[k]);
   };
   if (warp < kUWarps) {
     const int c = lane;
@@ -735,7 +838,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         }
         const int kq = q % nsub;
         const int rtl = q / nsub;
-        const int rt = blockIdx.y + rtl * G;
+        const int rt = g0 + rtl * G;
         mbar_expect_tx(&sh.qfull[b], static_cast<uint32_t>(kUBox));
         tma_load_2d(base + b * kUBox, &mapQ, &sh.qfull[b], rt * kUM, kq * kUS);
         if (b) ++nq1; else ++nq0;
@@ -807,6 +910,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     uint64_t alo[kCols], ahi[kCols];
     const uint64_t lo0 = 0 - static_cast<uint64_t>(gpt) * kReadLo;
     const uint64_t hi0 = 0 - static_cast<uint64_t>(gpt) * kReadHi;
+    const uint32_t one = blockDim.z;   // 1
 #pragma unroll
     for (int c = 0; c < kCols; ++c) { alo[c] = lo0; ahi[c] = hi0; }
     // level sums of the group ending at stage pq; the epilogue after a
@@ -826,7 +930,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         // epilogue of the row tile: X = beta X + alpha V' 2^(g_c - 68)
         if (loadx && !mbar_wait(&sh.xfull, static_cast<uint32_t>(rtl & 1))) sh.fail = 1;
         if (__any_sync(0xffffffffu, failed())) return false;
-        const int64_t r = (blockIdx.y + static_cast<int64_t>(rtl) * G) * kUM + m;
+        const int64_t r = (g0 + static_cast<int64_t>(rtl) * G) * kUM + m;
         const int c0 = n0 + cg * kCols;
         const double* xs = reinterpret_cast<const double*>(stX) + cg * kCols * kUM + m;
         double* xr = X + r + static_cast<int64_t>(c0) * ldx;
@@ -839,8 +943,8 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           double p;
           if (gcol < -2000) p = 0.0;
           else if (apow2) {
-            p = int96_to_double(hi, lo, gcol - 68 + ka - 1);
-            if (fa < 0.0) p = -p;
+            p = int96_to_double(hi, lo, gcol - 68 + ka);
+            p = __longlong_as_double(__double_as_longlong(p) ^ static_cast<long long>(asign));
           } else {
             p = int96_to_double(hi, lo, gcol - 68) * alpha;
           }
@@ -879,27 +983,39 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       const int k0 = kq * kUS + kCols * cg;
       if (kq * kUS + 16 * (cg >> 1) < i) {
         const unsigned char* col = base + b * kUBox + kCols * cg * 1024 + m * 8;
-        const int4 e0 = *reinterpret_cast<const int4*>(tb.eq + k0);
-        const int4 e1 = *reinterpret_cast<const int4*>(tb.eq + k0 + 4);
-        const int e8[kCols] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+        double v[kCols];
+        alignas(16) uint32_t w8[kCols];
+        uint32_t ta = 0xFFFFFFFFu;
+        *reinterpret_cast<uint4*>(w8) = *reinterpret_cast<const uint4*>(tb.w + k0);
+        *reinterpret_cast<uint4*>(w8 + 4) = *reinterpret_cast<const uint4*>(tb.w + k0 + 4);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t words[kDig][2];
-#pragma unroll
-          for (int w = 0; w < 2; ++w) {
-            const int c = 4 * h + 2 * w;
-            const double va = *reinterpret_cast<const double*>(col + c * 1024);
-            const double vb = *reinterpret_cast<const double*>(col + (c + 1) * 1024);
-            uint32_t d8[kDig];
-            cut_pair(va, e8[c], vb, e8[c + 1], d8);
-#pragma unroll
-            for (int t = 0; t < kDig; ++t) words[t][w] = d8[t];
-          }
-#pragma unroll
-          for (int t = 0; t < kDig; ++t)
-            tmem_st2(tlane + kUACol + static_cast<uint32_t>(128 * b + 16 * t + 4 * cg + 2 * h),
-                     words[t]);
+        for (int c = 0; c < kCols; ++c) {
+          v[c] = *reinterpret_cast<const double*>(col + c * 1024);
+          ta = min(ta, near_test(v[c], w8[c]));
         }
+        auto cut = [&](auto near) {
+          constexpr bool kNear = decltype(near)::value;
+          auto ex = [&](int c) { return k0 + c < i ? __ldg(eq + k0 + c) : -4000; };
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t words[kDig][2];
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+              const int c = 4 * h + 2 * w;
+              uint32_t d8[kDig];
+              if (kNear) cut_pair_near(v[c], w8[c], v[c + 1], w8[c + 1], one, d8);
+              else cut_pair(v[c], ex(c), v[c + 1], ex(c + 1), d8);
+#pragma unroll
+              for (int t = 0; t < kDig; ++t) words[t][w] = d8[t];
+            }
+#pragma unroll
+            for (int t = 0; t < kDig; ++t)
+              tmem_st2(tlane + kUACol + static_cast<uint32_t>(128 * b + 16 * t + 4 * cg + 2 * h),
+                       words[t]);
+          }
+        };
+        if (__all_sync(0xffffffffu, ta > kNearMin)) cut(std::true_type{});
+        else cut(std::false_type{});
       }
       mbar_arrive(&sh.qfree[b]);
       tmem_st_wait();
@@ -1645,13 +1761,10 @@ void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, 
   SG_REQUIRE(make_map64_box(&mq, Q, n, i, ldq) && make_map64_box(&mx, X, n, s, ldx), SG_ECUDA,
              "cuTensorMapEncodeTiled failed");
   ensure_dynamic_smem(reinterpret_cast<const void*>(oz_update_kernel), oz_update_smem(kUMaxK));
-  const int ct = (s + kUN - 1) / kUN;
+  const int64_t ct = (s + kUN - 1) / kUN;
   const int64_t ntiles = (n + kUM - 1) / kUM;
-  int64_t G = static_cast<int64_t>(device_sm_count()) / ct;
-  if (G < 1) G = 1;
-  if (G > ntiles) G = ntiles;
-  dim3 grid(static_cast<unsigned>(ct), static_cast<unsigned>(G));
-  oz_update_kernel<<<grid, kUThreads, oz_update_smem(i), st>>>(
+  const int64_t P = std::max<int64_t>(ct, std::min<int64_t>(device_sm_count(), ct * ntiles));
+  oz_update_kernel<<<static_cast<unsigned>(P), kUThreads, oz_update_smem(i), st>>>(
       mq, mx, n, i, s, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0, exps, err);
   SG_LAUNCH_CHECK();
   oz_check_error_pending.fetch_add(1);
