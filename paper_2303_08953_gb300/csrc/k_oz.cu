@@ -1300,10 +1300,25 @@ __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
   return d;
 }
 
-// grid: (quarters of 32 output columns, splits of the rows)
+// The rows are split separately for every quarter: quarter q's CTAs are
+// first[q] .. first[q + 1] - 1, each takes rows[q] rows, and the partials of
+// all quarters fill smax slots (zeros where a quarter has fewer splits).
+// The splits go by the time of a stage: with one split for all, quarter 0
+// (1.0 us a stage) waited for quarter 1 (1.4 us) or 3 (1.6 us).
+// Measured with the cut spread over the schedulers and the rows split so
+// (before in brackets): 2^21 rows, 20 columns 451 us (705), 120 columns
+// 2.42 ms (2.80); 2^20 rows, 60 columns 569 us (745).
+struct OzGramPlan {
+  int first[5];
+  int smax;
+  int64_t rows[4];
+};
+constexpr int kGWork[4] = {10, 14, 15, 16};
+
+// grid: the CTAs of every quarter of 32 output columns in turn
 __global__ void __launch_bounds__(kDThreads, 1)
 oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
-                 const int* __restrict__ ex, int64_t rows_per_split,
+                 const int* __restrict__ ex, const __grid_constant__ OzGramPlan plan,
                  double* __restrict__ part, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char dsmem[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
@@ -1311,9 +1326,12 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
-  const int q = blockIdx.x;
-  const int64_t k0 = static_cast<int64_t>(blockIdx.y) * rows_per_split;
-  const int64_t k1 = (k0 + rows_per_split < n) ? k0 + rows_per_split : n;
+  const int bx = static_cast<int>(blockIdx.x);
+  const int q = (bx >= plan.first[1]) + (bx >= plan.first[2]) + (bx >= plan.first[3]);
+  const int split = bx - plan.first[q];
+  const int nsplit = plan.first[q + 1] - plan.first[q];
+  const int64_t k0 = split * plan.rows[q];
+  const int64_t k1 = (k0 + plan.rows[q] < n) ? k0 + plan.rows[q] : n;
   const int nk = static_cast<int>((k1 - k0 + kGK - 1) / kGK);
   auto stage = [&](int r) { return base + r * kGStageBytes; };
   auto sliceA = [&](int b, int t) { return base + kGSlicesOff + b * kGBuf + kGAOff + t * kGSliceA; };
@@ -1322,20 +1340,28 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
   auto failed = [&]() { return *reinterpret_cast<volatile int*>(&sh.fail) != 0; };
   auto group_end = [&](int k) { return (k % kGChunk) == kGChunk - 1 || k == nk - 1; };
 
-  // warps 0-7 cut, warps 8-15 read out; of each, the two warps per group of
-  // 32 tensor-memory lanes whose lanes hold columns 0 .. 32q + 31 take part
-  // (the others wait at the end)
-  const uint32_t nwork = static_cast<uint32_t>(64 * (q + 1));
+  // Warps 0-7 cut, warps 8-15 read out.  The cut's units are a group of 32
+  // columns (a lane each) by 8 rows of the stage, unit u = columns
+  // 32 (u % (q + 1)) .. + 31, rows 8 (u / (q + 1)) .. + 7; warp w takes units
+  // w and w + 8, so that they are spread over all four schedulers whatever
+  // the quarter (tied to the tensor-memory lanes of their columns, the units
+  // of q = 0 ran on one scheduler and those of q = 1 on two: 1.6 us a stage
+  // for every quarter).  Of the reading warps, which reach only the lanes of
+  // their own scheduler, the two whose lanes hold columns 0 .. 32q + 31 take
+  // part per group of 32 columns (the others wait at the end).
+  const int nunits = 4 * (q + 1);
+  const uint32_t ncut = static_cast<uint32_t>(32 * (nunits < 8 ? nunits : 8));
+  const uint32_t nread = static_cast<uint32_t>(64 * (q + 1));
   if (tid == 0) {
     for (int r = 0; r < kGRing; ++r) {
       mbar_init(&sh.full[r], 1);
-      mbar_init(&sh.sfree[r], nwork);
+      mbar_init(&sh.sfree[r], ncut);
     }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(&sh.afull[b], nwork);
+      mbar_init(&sh.afull[b], ncut);
       mbar_init(&sh.afree[b], 1);
       mbar_init(&sh.accfull[b], 1);
-      mbar_init(&sh.accfree[b], nwork);
+      mbar_init(&sh.accfree[b], nread);
     }
     mbar_init(&sh.done, 1);
     sh.fail = 0;
@@ -1368,17 +1394,16 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = sh.tmem_base;
 
-  // Warp w (w < 16) covers the tensor-memory lanes, i.e. columns,
-  // m = 32 (w % 4) + lane; half = (w / 4) % 2.  A cutting warp (w < 8) cuts
-  // rows 16 half .. + 15 of each stage of column m; a reading warp (w >= 8)
-  // owns the outputs (m, 32q + 16 half + c), c < 16, each as two int64
-  // halves: ahi = sum of S_l 256^(3-l) over l = 0..3, alo = sum of
-  // S_l 256^(7-l) over l = 4..7 (|S_l| < 2^24: each half grows by < 2^48.1
-  // per readout and stays exact for 2^14 readouts); V = ahi 2^32 + alo
+  // A reading warp w covers the tensor-memory lanes, i.e. columns,
+  // m = 32 (w % 4) + lane; half = (w / 4) % 2; it owns the outputs
+  // (m, 32q + 16 half + c), c < 16, each as two int64 halves:
+  // ahi = sum of S_l 256^(3-l) over l = 0..3, alo = sum of S_l 256^(7-l)
+  // over l = 4..7 (|S_l| < 2^24: each half grows by < 2^48.1 per readout and
+  // stays exact for 2^14 readouts); V = ahi 2^32 + alo
   const int m = (warp & 3) * 32 + lane;
   const int half = (warp >> 2) & 1;
-  const bool mine = (warp & 3) <= q;   // columns 32 (w % 4) .. + 31 are within 0 .. 32q + 31
   const bool cutter = warp < kDWarps / 2;
+  const bool mine = cutter ? warp < nunits : (warp & 3) <= q;
   uint64_t alo[16];
   uint64_t ahi[16];
   const uint64_t reads = static_cast<uint64_t>((nk + kGChunk - 1) / kGChunk);
@@ -1465,14 +1490,24 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
     }
   } else if (mine && cutter) {
     // ------------------------------------------------ cut
-    const int em = m < s ? ex[m] : -4000;
     // u = x 2^(6 - e) as two exact power-of-two scalings, both factors
     // normal; columns that are all zero, beyond s or hold an Inf or a NaN
     // are cut as zeros
-    const bool live = em > -2000 && em < kGNonFinite;
-    const int eb = (live && em < -50) ? 64 : 0;
-    const float f1 = __int_as_float((127 + eb) << 23);
-    const float f2 = live ? __int_as_float((127 + 6 - em - eb) << 23) : 0.0f;
+    const int units = warp + 8 < nunits ? 2 : 1;
+    int col[2], chunk[2];
+    bool live[2];
+    float f1[2], f2[2];
+#pragma unroll
+    for (int gg = 0; gg < 2; ++gg) {
+      const int u = warp + 8 * gg;
+      col[gg] = kGN * (u % (q + 1)) + lane;
+      chunk[gg] = u / (q + 1);
+      const int em = u < nunits && col[gg] < s ? ex[col[gg]] : -4000;
+      live[gg] = em > -2000 && em < kGNonFinite;
+      const int eb = (live[gg] && em < -50) ? 64 : 0;
+      f1[gg] = __int_as_float((127 + eb) << 23);
+      f2[gg] = live[gg] ? __int_as_float((127 + 6 - em - eb) << 23) : 0.0f;
+    }
     constexpr float kRound = 12582912.0f;   // 1.5 2^23: adding it rounds |v| < 2^22 to an integer
     for (int k = 0; k < nk; ++k) {
       const int b = k & 1;
@@ -1489,9 +1524,10 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
       if (__any_sync(0xffffffffu, bad)) break;
 #pragma unroll
       for (int gg = 0; gg < 2; ++gg) {
-        // column m's rows 8 cg .. + 7 (cg = 2 half + gg): chunks 2 cg,
-        // 2 cg + 1 of its 128-byte swizzled line in the staged boxes
-        const int cg = 2 * half + gg;
+        if (gg >= units) break;
+        // column m's rows 8 cg .. + 7: chunks 2 cg, 2 cg + 1 of its 128-byte
+        // swizzled line in the staged boxes
+        const int m = col[gg], cg = chunk[gg];
         const unsigned char* line = stage(r) + m * 128;
         const uint4 r0 = *reinterpret_cast<const uint4*>(line + (((2 * cg) ^ (m & 7)) << 4));
         const uint4 r1 = *reinterpret_cast<const uint4*>(line + (((2 * cg + 1) ^ (m & 7)) << 4));
@@ -1500,8 +1536,8 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
           // rows 2p (low half) and 2p + 1 (high half) of the word
-          float ua = live ? __fmul_rn(__fmul_rn(__uint_as_float(v[2 * p]), f1), f2) : 0.0f;
-          float ub = live ? __fmul_rn(__fmul_rn(__uint_as_float(v[2 * p + 1]), f1), f2) : 0.0f;
+          float ua = live[gg] ? __fmul_rn(__fmul_rn(__uint_as_float(v[2 * p]), f1[gg]), f2[gg]) : 0.0f;
+          float ub = live[gg] ? __fmul_rn(__fmul_rn(__uint_as_float(v[2 * p + 1]), f1[gg]), f2[gg]) : 0.0f;
 #pragma unroll
           for (int t = 0; t < kGDig; ++t) {
             const float da = __fsub_rn(__fadd_rn(ua, kRound), kRound);
@@ -1523,7 +1559,7 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
         for (int t = 0; t < kGDig; ++t)
           *reinterpret_cast<uint4*>(dst + t * kGSliceA) =
               make_uint4(words[t][0], words[t][1], words[t][2], words[t][3]);
-        if ((warp & 3) == q) {
+        if ((m >> 5) == q) {
           unsigned char* dstb = sliceB(b, 0) + lane * 64 + off;
 #pragma unroll
           for (int t = 0; t < kGDig; ++t)
@@ -1550,7 +1586,7 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
   if (!good) {
     if (tid == 0) atomicExch(err, 1);
   } else if (warp < kDWarps && !cutter && mine && m < s) {
-    double* P = part + static_cast<int64_t>(blockIdx.y) * s * s;
+    double* P = part + static_cast<int64_t>(split) * s * s;
     const int em = ex[m];
 #pragma unroll
     for (int cc = 0; cc < 16; ++cc) {
@@ -1569,6 +1605,8 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
           val = int96_to_double(hi, lo, em + en - 68);
         }
         P[m + static_cast<int64_t>(nn) * s] = val;
+        for (int z = split + nsplit; z < plan.smax; z += nsplit)
+          P[static_cast<int64_t>(z - split) * s * s + m + static_cast<int64_t>(nn) * s] = 0.0;
       }
     }
   }
@@ -1666,20 +1704,27 @@ bool make_map32_gram(CUtensorMap* map, const float* ptr, int64_t rows, int64_t c
          CUDA_SUCCESS;
 }
 
-int64_t oz_gram32_splits(int64_t n, int s, int64_t* rows) {
-  const int64_t nq = (s + kGN - 1) / kGN;
-  int64_t S = static_cast<int64_t>(device_sm_count()) / nq;
-  const int64_t maxS = n / (4 * kGK);     // at least four stages per split
-  if (S > maxS) S = maxS;
-  // at most 2^14 level readouts per split keep the int64 halves exact
+OzGramPlan oz_gram32_plan(int64_t n, int s) {
+  OzGramPlan p{};
+  const int nq = (s + kGN - 1) / kGN;
+  int all = 0;
+  for (int q = 0; q < nq; ++q) all += kGWork[q];
+  // at least four stages per split; at most 2^14 level readouts per split
+  // keep the int64 halves exact
+  const int64_t maxS = n / (4 * kGK);
   const int64_t span = int64_t(kGK) * kGChunk << 14;
   const int64_t minS = (n + span - 1) / span;
-  if (S < minS) S = minS;
-  if (S < 1) S = 1;
-  int64_t r = (n + S - 1) / S;
-  r = (r + kGK - 1) / kGK * kGK;
-  if (rows) *rows = r;
-  return (n + r - 1) / r;
+  for (int q = 0; q < nq; ++q) {
+    int64_t S = static_cast<int64_t>(device_sm_count()) * kGWork[q] / all;
+    S = std::max<int64_t>({std::min(S, maxS), minS, 1});
+    const int64_t r = ((n + S - 1) / S + kGK - 1) / kGK * kGK;
+    const int c = static_cast<int>((n + r - 1) / r);
+    p.rows[q] = r;
+    p.first[q + 1] = p.first[q] + c;
+    p.smax = std::max(p.smax, c);
+  }
+  for (int q = nq; q < 4; ++q) p.first[q + 1] = p.first[nq];
+  return p;
 }
 
 }  // namespace
@@ -1815,40 +1860,37 @@ bool oz_gram32_supported(int64_t n, const float* X, int64_t ldx, int s) {
 }
 
 // Expected time of the tensor-core Gram: one CTA per SM takes a quarter of
-// 32 output columns through stages of 32 rows at about kStageUs each
-// (measured 1.6 us at n = 2^19 .. 2^21, s = 16 .. 128, whatever the
-// quarter: a warp reaches the tensor-memory lanes of its own scheduler
-// only, so each group of 32 columns is read out, and its columns cut, by
-// one scheduler's warps, and their instruction issue, not the MMAs, sets
-// the pace), plus kFixedUs of setup (the exponent and reduction launches,
-// tensor memory).
+// 32 output columns through stages of 32 rows at kGWork / 10 times about
+// kStageUs each (measured 1.0 us for quarter 0, about what its MMAs take,
+// to 1.6 us for quarter 3), the quarters' CTAs shared out by that, plus
+// kFixedUs of setup (the exponent and reduction launches, tensor memory).
 double oz_gram32_seconds(int64_t n, int s) {
-  constexpr double kStageUs = 1.6, kFixedUs = 15.0;
-  const double nq = static_cast<double>((s + kGN - 1) / kGN);
-  return (static_cast<double>((n + kGK - 1) / kGK) * nq * kStageUs /
+  constexpr double kStageUs = 1.0, kFixedUs = 15.0;
+  double work = 0.0;
+  for (int q = 0; q * kGN < s; ++q) work += kGWork[q] / 10.0;
+  return (static_cast<double>((n + kGK - 1) / kGK) * work * kStageUs /
               static_cast<double>(device_sm_count()) +
           kFixedUs) * 1e-6;
 }
 
 int64_t oz_gram32_part_size(int64_t n, int s) {
-  return oz_gram32_splits(n, s, nullptr) * s * s;
+  return static_cast<int64_t>(oz_gram32_plan(n, s).smax) * s * s;
 }
 
 void oz_gram32(int64_t n, const float* X, int64_t ldx, int s, int* exps, double* part,
                int64_t part_cap, int* nsplit, cudaStream_t st) {
   int* err = oz_err_flag();
-  int64_t rows = 0;
-  const int64_t S = oz_gram32_splits(n, s, &rows);
-  SG_REQUIRE(S * s * s <= part_cap, SG_EINVAL, "oz_gram32: workspace too small");
+  const OzGramPlan plan = oz_gram32_plan(n, s);
+  SG_REQUIRE(static_cast<int64_t>(plan.smax) * s * s <= part_cap, SG_EINVAL,
+             "oz_gram32: workspace too small");
   col_exponents32(n, X, ldx, s, exps, st);
   CUtensorMap mx;
   SG_REQUIRE(make_map32_gram(&mx, X, n, s, ldx), SG_ECUDA, "cuTensorMapEncodeTiled failed");
   ensure_dynamic_smem(reinterpret_cast<const void*>(oz_gram32_kernel), kGSmem);
-  dim3 grid((s + kGN - 1) / kGN, static_cast<unsigned>(S));
-  oz_gram32_kernel<<<grid, kDThreads, kGSmem, st>>>(mx, n, s, exps, rows, part, err);
+  oz_gram32_kernel<<<plan.first[4], kDThreads, kGSmem, st>>>(mx, n, s, exps, plan, part, err);
   SG_LAUNCH_CHECK();
   oz_check_error_pending.fetch_add(1);
-  *nsplit = static_cast<int>(S);
+  *nsplit = plan.smax;
 }
 
 }  // namespace sg
