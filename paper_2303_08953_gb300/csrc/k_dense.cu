@@ -19,6 +19,7 @@
 // a two-sum, so the Gram of FP32 vectors is accurate to about eps_32^2
 // relative to the sum of |products| -- the accuracy the partial Cholesky
 // bound of the FP32 basis relies on.
+#include <algorithm>
 #include <atomic>
 #include <cstdlib>
 
@@ -40,7 +41,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 
 // C_part[z] (M x N, column-major) = A(k0:k1, :)^T B(k0:k1, :)
 // Tile BM x BN, thread tile TM x TN; MW: thread rows vary across warps
-// (whole warps idle on padded rows).
+// (whole warps idle on padded rows, otherwise on padded columns).
 template <int BM, int BN, int TM, int TN, bool MW, bool EXACT, typename T>
 __global__ void __launch_bounds__(kThreads)
 dot_tile_kernel(int64_t K, int M, int N, const T* __restrict__ A,
@@ -58,7 +59,7 @@ dot_tile_kernel(int64_t K, int M, int N, const T* __restrict__ A,
   const int tid = threadIdx.x;
   const int tx = MW ? tid / TNN : tid % TMN;
   const int ty = MW ? tid % TNN : tid / TMN;
-  const bool active = (m0 + tx * TM) < M;
+  const bool active = (m0 + tx * TM) < M && (n0 + ty * TN) < N;
   T acc[TM][TN], comp[TM][TN];
 #pragma unroll
   for (int a = 0; a < TM; ++a)
@@ -235,6 +236,30 @@ void launch_reduce(int M, int N, int S, const double* part, double* W, int ldw,
   SG_LAUNCH_CHECK();
 }
 
+// The most row splits a block dot of `tiles` CTAs per split may have: at
+// least four stages of BK rows each, but down to one while two CTAs per SM
+// are not reached (n = 4096, s = 10, the average over i = 11 .. 25: 32 CTAs
+// took 20.1 us, 128 take 7.1; 16 x 16 tiles for i up to 51: 18.0 -> 9.5).
+int64_t max_splits(int64_t n, int64_t tiles) {
+  const int64_t fill = (2 * static_cast<int64_t>(device_sm_count()) + tiles - 1) / tiles;
+  return std::max((n + 4 * BK - 1) / (4 * BK), std::min((n + BK - 1) / BK, fill));
+}
+
+// Whether the one-thread-per-output kernel takes an FP64 product, its
+// outputs, and its row splits.
+bool small_dot(int i, int s, bool sym) {
+  return i + s <= kSmallCols &&
+         (sym && i == s ? s * (s + 1) / 2 <= kSmallOut : (i > 8 && i * s <= kSmallOut));
+}
+
+int64_t small_splits(int64_t n, int nout) {
+  const int threads = (nout + 31) / 32 * 32;
+  int64_t S = static_cast<int64_t>(device_sm_count()) * (2048 / threads);
+  const int64_t maxS = max_splits(n, 1);
+  if (S > maxS) S = maxS;
+  return S < 1 ? 1 : S;
+}
+
 // Gram matrix of FP32 vectors, G = X^T X, with the products of the
 // EXACT path (p = a b rounded plus its FMA remainder, two-sum accumulation)
 // but without the square tiles' waste: a thread owns one 4 x 4 block
@@ -399,7 +424,7 @@ DotPlan plan_dot(int64_t n, int i, int s, bool wide, bool sym) {
                                   : static_cast<int64_t>(p.tm) * p.tn;
   const int64_t slots = static_cast<int64_t>(device_sm_count()) * (2048 / kThreads);
   int64_t S = slots / tiles;
-  const int64_t maxS = (n + 4 * BK - 1) / (4 * BK);  // >= 4 stages per split
+  const int64_t maxS = max_splits(n, tiles);
   if (S > maxS) S = maxS;
   if (S < 1) S = 1;
   if (S > 4096) S = 4096;
@@ -482,17 +507,13 @@ void block_dot_impl(int64_t n, const T* Q, int64_t ldq, int i, const T* X,
     launch_reduce(i, s, S, part, W, ldw, false, st);
     return;
   }
-  if (sizeof(T) == 8 && i + s <= kSmallCols &&
-      (sym && i == s ? s * (s + 1) / 2 <= kSmallOut : (i > 8 && i * s <= kSmallOut))) {
+  if (sizeof(T) == 8 && small_dot(i, s, sym)) {
     // small FP64 products: one thread per needed output (a Q of at most
     // eight columns keeps the narrow tile, whose idle rows are whole warps)
     const bool tri = sym && i == s;
     const int nout = tri ? s * (s + 1) / 2 : i * s;
     const int threads = (nout + 31) / 32 * 32;
-    int64_t S = static_cast<int64_t>(device_sm_count()) * (2048 / threads);
-    const int64_t maxS = (n + 4 * BK - 1) / (4 * BK);
-    if (S > maxS) S = maxS;
-    if (S < 1) S = 1;
+    int64_t S = small_splits(n, nout);
     if (S * i * s > part_cap) S = part_cap / (static_cast<int64_t>(i) * s);
     SG_REQUIRE(S >= 1, SG_EINVAL, "block_dot: workspace too small");
     int64_t rows = (n + S - 1) / S;
@@ -655,6 +676,7 @@ update_kernel(int64_t K, int M, int N, const T* __restrict__ A, int64_t lda,
 #pragma unroll
     for (int b = 0; b < TN; ++b) acc[a][b] = T(0);
   const int mend = upper ? ((n0 + UN < M) ? n0 + UN : M) : M;
+  const bool active = n0 + ty * TN < N;     // ty varies across warps: whole warps idle
   for (int mb = 0; mb < mend; mb += UK) {
     for (int e = tid; e < UK * UR; e += kThreads) {
       const int rr = e % UR, mm = e / UR;
@@ -672,6 +694,8 @@ update_kernel(int64_t K, int M, int N, const T* __restrict__ A, int64_t lda,
     __syncthreads();
 #pragma unroll
     for (int mm = 0; mm < UK; ++mm) {
+      // padding would cost the FP64 pipe as much as the product itself
+      if (!active || (sizeof(T) == 8 && mb + mm >= mend)) break;
       T av[TR], bv[TN];
 #pragma unroll
       for (int a = 0; a < TR; ++a) av[a] = As[mm][tx * TR + a];
@@ -836,9 +860,19 @@ void block_update_impl(int64_t n, const T* Q, int64_t ldq, int i,
     update_kernel<128, 8, 4, 1, T><<<grid, kThreads, 0, st>>>(
         n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
   } else if (sizeof(T) == 8) {
-    dim3 grid(static_cast<unsigned>((n + 63) / 64), (s + 15) / 16);
-    update_kernel<64, 16, 4, 1, T><<<grid, kThreads, 0, st>>>(
-        n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
+    // 64 rows per CTA, 32 where that makes fewer than two CTAs per SM
+    // (n = 4096, s = 10, the average over i = 21 .. 51: 19.5 -> 9.6 us, idle
+    // columns and inner padding left out included)
+    const int64_t cols = (s + 15) / 16, r64 = (n + 63) / 64;
+    if (r64 * cols < 2 * static_cast<int64_t>(device_sm_count())) {
+      dim3 grid(static_cast<unsigned>((n + 31) / 32), static_cast<unsigned>(cols));
+      update_kernel<32, 16, 2, 1, T><<<grid, kThreads, 0, st>>>(
+          n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
+    } else {
+      dim3 grid(static_cast<unsigned>(r64), static_cast<unsigned>(cols));
+      update_kernel<64, 16, 4, 1, T><<<grid, kThreads, 0, st>>>(
+          n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
+    }
   } else if (s <= 32) {
     // FP32, narrow blocks: 128 x 32 tiles, 4 x 4 outputs per thread
     dim3 grid(static_cast<unsigned>((n + 127) / 128), 1);
@@ -898,6 +932,8 @@ int64_t block_dot_part_size(int64_t n, int i, int s) {
       const DotPlan a = plan_dot(n, i, s, w == 1, y == 1);
       if (a.S > S) S = a.S;
     }
+  if (small_dot(i, s, false)) S = std::max(S, small_splits(n, i * s));
+  if (small_dot(i, s, true)) S = std::max(S, small_splits(n, i == s ? s * (s + 1) / 2 : i * s));
   int64_t need = S * i * s;
   if (i == s && s <= kGramMaxS) {
     int64_t g = gram_splits(n, s, nullptr) * s * s;

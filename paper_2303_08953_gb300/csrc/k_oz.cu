@@ -696,7 +696,7 @@ int oz_update_smem(int i) {
 // P >= ntc: at least one each, the rest in proportion to the tile's work, a
 // fixed part (readout, epilogue) and its 16-column steps of Q.  With W upper
 // triangular, column tile ct needs only Q's columns 0 .. 32 ct + 31.
-constexpr int kUTileW = 6;                              // fixed part, in steps
+constexpr int kUTileW = 7;                              // fixed part, in steps
 
 __host__ __device__ inline int oz_update_first(int ct, int ntc, int i, int upper, int P) {
   int64_t before = 0, all = 0;
@@ -1740,20 +1740,20 @@ bool oz_dot_supported(int64_t n, const double* Q, int64_t ldq, int i, const doub
 
 // Whether the tensor-core form is expected to beat the FP64-pipe kernel:
 // a tile of 128 x 32 outputs costs about kStageUs per 32 rows on one SM
-// (measured 2.2 .. 2.4 us over i = 13 .. 240) plus kFixedUs of setup (the
-// exponent and reduction launches, barriers, tensor memory), the FP64-pipe
-// kernels about
-// 1 TFLOP/s (2 n i s flops; the symmetric Gram n s (s+1)) plus their
-// streams of Q and X at about 2 TB/s.
+// (measured 1.75 .. 1.85 us over i = 13 .. 241, s = 12 .. 120 at 2^21 rows),
+// the exponents read Q and X once more at about 6 TB/s, plus kFixedUs of
+// setup (the exponent and reduction launches, barriers, tensor memory); the
+// FP64-pipe kernels about 1 TFLOP/s (2 n i s flops; the symmetric Gram
+// n s (s+1)) plus their streams of Q and X at about 2 TB/s.
 bool oz_dot_pays(int64_t n, int i, int s, bool sym) {
-  constexpr double kStageUs = 2.4, kFixedUs = 15.0;
+  constexpr double kStageUs = 1.8, kFixedUs = 15.0;
   const double tiles = static_cast<double>((i + kOM - 1) / kOM) * ((s + kON - 1) / kON);
-  const double t_oz = (static_cast<double>((n + kOK - 1) / kOK) * tiles * kStageUs /
-                           static_cast<double>(device_sm_count()) +
-                       kFixedUs) * 1e-6;
   const double flops = sym ? static_cast<double>(n) * s * (s + 1.0)
                            : 2.0 * static_cast<double>(n) * i * s;
   const double bytes = static_cast<double>(n) * (sym ? s : i + s) * 8.0;
+  const double t_oz = (static_cast<double>((n + kOK - 1) / kOK) * tiles * kStageUs /
+                           static_cast<double>(device_sm_count()) +
+                       kFixedUs) * 1e-6 + bytes / 6.0e12;
   return t_oz < 0.9 * (flops / 1.0e12 + bytes / 2.0e12);
 }
 
@@ -1773,23 +1773,27 @@ bool oz_update_supported(int64_t n, const double* Q, int64_t ldq, int i, const d
 }
 
 // Whether the tensor-core update is expected to beat the FP64-pipe kernel.
-// One SM takes ceil(row tiles / row groups) tiles of 128 rows x 32 columns,
-// each about kTileUs (readout, epilogue, pipeline fill) plus kStepUs per
-// 16 columns of Q (measured: 7.7 us at 1 step, 14.6 us at 7, 23.4 us at 15),
-// plus kFixedUs of setup (the exponent launch, W's digits, tensor memory).
+// One SM takes its share of the tiles of 128 rows x 32 columns, each about
+// kTileUs (readout, epilogue, pipeline fill) plus kStepUs per 16 columns of
+// Q (measured: 6.5 us at 1 step, 8.1 us at 4, 10.1 us at 8, 16.8 us at 16),
+// with W upper triangular only those down to the diagonal; the exponents
+// read Q once more at about 6 TB/s; plus kFixedUs of setup (the exponent
+// launch, W's digits, tensor memory).
 // The FP64-pipe kernels sustain about 1.05 TFLOP/s (2 n i s flops, half
 // for the triangle); the tiled one adds its streams of Q and X at about
 // 2 TB/s, the narrow-Q one (i <= 16) overlaps them at about 5.5 TB/s.
 bool oz_update_pays(int64_t n, int i, int s, bool upper) {
-  constexpr double kTileUs = 6.6, kStepUs = 1.12, kFixedUs = 15.0;
+  constexpr double kTileUs = 5.2, kStepUs = 0.72, kFixedUs = 15.0;
   const int64_t ct = (s + kUN - 1) / kUN;
   const int64_t ntiles = (n + kUM - 1) / kUM;
-  int64_t G = static_cast<int64_t>(device_sm_count()) / ct;
-  if (G < 1) G = 1;
-  if (G > ntiles) G = ntiles;
-  const double per_sm = static_cast<double>((ntiles + G - 1) / G) *
-                        ((ct + device_sm_count() - 1) / device_sm_count());
-  const double t_oz = (per_sm * (kTileUs + kStepUs * ((i + 15) / 16)) + kFixedUs) * 1e-6;
+  const int64_t P = std::max<int64_t>(ct, std::min<int64_t>(device_sm_count(), ct * ntiles));
+  double row = 0.0;   // the tiles of one row of tiles
+  for (int64_t c = 0; c < ct; ++c) {
+    const int64_t k = upper ? std::min<int64_t>(i, (c + 1) * kUN) : i;
+    row += kTileUs + kStepUs * static_cast<double>((k + 15) / 16);
+  }
+  const double per_sm = static_cast<double>((ntiles * ct + P - 1) / P) / static_cast<double>(ct);
+  const double t_oz = (per_sm * row + kFixedUs) * 1e-6 + static_cast<double>(n) * i * 8.0 / 6.0e12;
   const double flops = (upper ? 1.0 : 2.0) * static_cast<double>(n) * i * s;
   const double bytes = static_cast<double>(n) * (i + 2.0 * s) * 8.0;
   const double t_fp64 = i <= 16 ? std::max(flops / 1.05e12, bytes / 5.5e12)
