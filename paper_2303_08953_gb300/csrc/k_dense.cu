@@ -23,6 +23,7 @@
 #include <atomic>
 #include <cstdlib>
 
+#include "k_launch.cuh"
 #include "sg_internal.h"
 
 namespace sg {
@@ -50,6 +51,8 @@ dot_tile_kernel(int64_t K, int M, int N, const T* __restrict__ A,
   constexpr bool kF32 = sizeof(T) == 4;
   constexpr int TMN = BM / TM, TNN = BN / TN;
   static_assert(TMN * TNN == kThreads, "thread layout");
+  wait_previous();
+  release_next();
   if (sym && blockIdx.x > blockIdx.y) return;
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
   const int64_t k0 = blockIdx.z * rows_per_split;
@@ -164,6 +167,8 @@ __global__ void __launch_bounds__(kSmallOut)
 dot_small_kernel(int64_t K, int M, int N, const double* __restrict__ A, int64_t lda,
                  const double* __restrict__ B, int64_t ldb, double* __restrict__ part,
                  int64_t rows_per_split, int sym) {
+  wait_previous();
+  release_next();
   extern __shared__ double small_smem[];
   double* As = small_smem;                     // BK x (M + 1)
   double* Bs = small_smem + BK * (M + 1);      // BK x (N + 1)
@@ -213,6 +218,8 @@ dot_small_kernel(int64_t K, int M, int N, const double* __restrict__ A, int64_t 
 __global__ void reduce_parts_kernel(int M, int N, int S,
                                     const double* __restrict__ part,
                                     double* __restrict__ W, int ldw, int sym) {
+  wait_previous();
+  release_next();
   const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (gw >= static_cast<int64_t>(M) * N) return;
@@ -231,8 +238,8 @@ __global__ void reduce_parts_kernel(int M, int N, int S,
 void launch_reduce(int M, int N, int S, const double* part, double* W, int ldw,
                    bool sym, cudaStream_t st) {
   const int64_t threads = static_cast<int64_t>(M) * N * 32;
-  reduce_parts_kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, st>>>(
-      M, N, S, part, W, ldw, sym ? 1 : 0);
+  launch_early(true, reduce_parts_kernel, dim3(static_cast<unsigned>((threads + 255) / 256)), 256, 0,
+               st, M, N, S, part, W, ldw, sym ? 1 : 0);
   SG_LAUNCH_CHECK();
 }
 
@@ -445,20 +452,20 @@ void launch_dot(const DotPlan& p, cudaStream_t st, int64_t n, int i, int s,
   const int sy = sym ? 1 : 0;
   switch (p.cfg) {
     case CFG_NARROW_M:
-      dot_tile_kernel<8, 32, 1, 1, true, EXACT, T><<<grid, kThreads, 0, st>>>(
-          n, i, s, Q, ldq, X, ldx, part, p.rows, 0);
+      launch_early(fills_once(grid), dot_tile_kernel<8, 32, 1, 1, true, EXACT, T>, grid, kThreads,
+                   0, st, n, i, s, Q, ldq, X, ldx, part, p.rows, 0);
       break;
     case CFG_NARROW_N:
-      dot_tile_kernel<64, 8, 2, 1, false, EXACT, T><<<grid, kThreads, 0, st>>>(
-          n, i, s, Q, ldq, X, ldx, part, p.rows, 0);
+      launch_early(fills_once(grid), dot_tile_kernel<64, 8, 2, 1, false, EXACT, T>, grid, kThreads,
+                   0, st, n, i, s, Q, ldq, X, ldx, part, p.rows, 0);
       break;
     case CFG_SQ16:
-      dot_tile_kernel<16, 16, 1, 1, false, EXACT, T><<<grid, kThreads, 0, st>>>(
-          n, i, s, Q, ldq, X, ldx, part, p.rows, sy);
+      launch_early(fills_once(grid), dot_tile_kernel<16, 16, 1, 1, false, EXACT, T>, grid, kThreads,
+                   0, st, n, i, s, Q, ldq, X, ldx, part, p.rows, sy);
       break;
     default:
-      dot_tile_kernel<32, 32, 2, 2, false, EXACT, T><<<grid, kThreads, 0, st>>>(
-          n, i, s, Q, ldq, X, ldx, part, p.rows, sy);
+      launch_early(fills_once(grid), dot_tile_kernel<32, 32, 2, 2, false, EXACT, T>, grid, kThreads,
+                   0, st, n, i, s, Q, ldq, X, ldx, part, p.rows, sy);
   }
   SG_LAUNCH_CHECK();
 }
@@ -520,7 +527,9 @@ void block_dot_impl(int64_t n, const T* Q, int64_t ldq, int i, const T* X,
     rows = (rows + BK - 1) / BK * BK;
     S = (n + rows - 1) / rows;
     const size_t smem = sizeof(double) * BK * (i + 1 + s + 1);
-    dot_small_kernel<<<static_cast<unsigned>(S), threads, smem, st>>>(
+    const dim3 grid(static_cast<unsigned>(S));
+    launch_early(
+        fills_once(grid), dot_small_kernel, grid, threads, smem, st,
         n, i, s, reinterpret_cast<const double*>(Q), ldq, reinterpret_cast<const double*>(X),
         ldx, part, rows, tri ? 1 : 0);
     SG_LAUNCH_CHECK();
@@ -662,6 +671,8 @@ __global__ void __launch_bounds__(kThreads)
 update_kernel(int64_t K, int M, int N, const T* __restrict__ A, int64_t lda,
               const double* __restrict__ B, int ldb, T* __restrict__ C,
               int64_t ldc, double alpha, double beta, int upper) {
+  wait_previous();
+  release_next();
   constexpr int TRN = UR / TR, TNN = UN / TN;
   static_assert(TRN * TNN == kThreads, "thread layout");
   const int64_t r0 = static_cast<int64_t>(blockIdx.x) * UR;
@@ -744,6 +755,8 @@ __global__ void __launch_bounds__(kThreads)
 update_thin_kernel(int64_t n, int i, int s, const T* __restrict__ Q, int64_t ldq,
                    const double* __restrict__ W, int ldw, T* __restrict__ X, int64_t ldx,
                    double alpha, double beta, int upper) {
+  wait_previous();
+  release_next();
   __shared__ T Ws[MAXI][kThinCols];
   const int c0 = blockIdx.y * kThinCols;
   const int cn = (s - c0 < kThinCols) ? s - c0 : kThinCols;
@@ -809,14 +822,14 @@ void launch_update_thin_i(dim3 grid, int64_t n, const T* Q, int64_t ldq, int i, 
                           int ldw, T* X, int64_t ldx, int s, double alpha, double beta, int up,
                           cudaStream_t st) {
   if (alpha == -1.0 && beta == 1.0)
-    update_thin_kernel<MAXI, 1, T><<<grid, kThreads, 0, st>>>(n, i, s, Q, ldq, W, ldw, X, ldx,
-                                                               alpha, beta, up);
+    launch_early(fills_once(grid), update_thin_kernel<MAXI, 1, T>, grid, kThreads, 0, st, n, i, s, Q,
+                 ldq, W, ldw, X, ldx, alpha, beta, up);
   else if (beta == 0.0)
-    update_thin_kernel<MAXI, 2, T><<<grid, kThreads, 0, st>>>(n, i, s, Q, ldq, W, ldw, X, ldx,
-                                                               alpha, beta, up);
+    launch_early(fills_once(grid), update_thin_kernel<MAXI, 2, T>, grid, kThreads, 0, st, n, i, s, Q,
+                 ldq, W, ldw, X, ldx, alpha, beta, up);
   else
-    update_thin_kernel<MAXI, 0, T><<<grid, kThreads, 0, st>>>(n, i, s, Q, ldq, W, ldw, X, ldx,
-                                                               alpha, beta, up);
+    launch_early(fills_once(grid), update_thin_kernel<MAXI, 0, T>, grid, kThreads, 0, st, n, i, s, Q,
+                 ldq, W, ldw, X, ldx, alpha, beta, up);
 }
 
 template <typename T>
@@ -857,8 +870,8 @@ void block_update_impl(int64_t n, const T* Q, int64_t ldq, int i,
   }
   if (s <= 8) {
     dim3 grid(static_cast<unsigned>((n + 127) / 128), 1);
-    update_kernel<128, 8, 4, 1, T><<<grid, kThreads, 0, st>>>(
-        n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
+    launch_early(fills_once(grid), update_kernel<128, 8, 4, 1, T>, grid, kThreads,
+                 0, st, n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
   } else if (sizeof(T) == 8) {
     // 64 rows per CTA, 32 where that makes fewer than two CTAs per SM
     // (n = 4096, s = 10, the average over i = 21 .. 51: 19.5 -> 9.6 us, idle
@@ -866,18 +879,18 @@ void block_update_impl(int64_t n, const T* Q, int64_t ldq, int i,
     const int64_t cols = (s + 15) / 16, r64 = (n + 63) / 64;
     if (r64 * cols < 2 * static_cast<int64_t>(device_sm_count())) {
       dim3 grid(static_cast<unsigned>((n + 31) / 32), static_cast<unsigned>(cols));
-      update_kernel<32, 16, 2, 1, T><<<grid, kThreads, 0, st>>>(
-          n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
+      launch_early(fills_once(grid), update_kernel<32, 16, 2, 1, T>, grid, kThreads,
+                 0, st, n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
     } else {
       dim3 grid(static_cast<unsigned>(r64), static_cast<unsigned>(cols));
-      update_kernel<64, 16, 4, 1, T><<<grid, kThreads, 0, st>>>(
-          n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
+      launch_early(fills_once(grid), update_kernel<64, 16, 4, 1, T>, grid, kThreads,
+                 0, st, n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
     }
   } else if (s <= 32) {
     // FP32, narrow blocks: 128 x 32 tiles, 4 x 4 outputs per thread
     dim3 grid(static_cast<unsigned>((n + 127) / 128), 1);
-    update_kernel<128, 32, 4, 4, T><<<grid, kThreads, 0, st>>>(
-        n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
+    launch_early(fills_once(grid), update_kernel<128, 32, 4, 4, T>, grid, kThreads,
+                 0, st, n, ii, s, Q, ldq, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0);
   } else {
     dim3 grid(static_cast<unsigned>((n + WR - 1) / WR), (s + WN - 1) / WN);
     update_wide_kernel<<<grid, kThreads, 0, st>>>(

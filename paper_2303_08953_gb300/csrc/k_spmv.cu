@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "k_reduce.cuh"
+#include "k_launch.cuh"
 #include "sg_internal.h"
 
 namespace sg {
@@ -196,6 +197,8 @@ sell_kernel(int n, int64_t rows32, const int* __restrict__ sptr,
             const uint16_t* __restrict__ soff, const int* __restrict__ sperm,
             const T* __restrict__ sval, const T* __restrict__ x, const T* __restrict__ z,
             T* __restrict__ y, T theta, T c, T inv_gamma) {
+  wait_previous();
+  release_next();
   for (int64_t pos = blockIdx.x * static_cast<int64_t>(kThreads) + threadIdx.x; pos < rows32;
        pos += static_cast<int64_t>(gridDim.x) * kThreads) {
     const int64_t row = PERM ? static_cast<int64_t>(__ldg(sperm + pos)) : pos;
@@ -241,8 +244,8 @@ void dispatch(const DevCsr& A, const T* val, const T* sval, const T* x, const T*
     const int g = static_cast<int>(blocks < 1 ? 1 : blocks);
     const T ig = T(1) / gamma;
     auto go = [&](auto kernel) {
-      kernel<<<g, kThreads, 0, st>>>(A.n, rows32, A.sptr, A.scol, A.sbase, A.soff, A.sperm, sval, x,
-                                     z, y, theta, c, ig);
+      launch_early(true, kernel, g, kThreads, 0, st, A.n, rows32, A.sptr, A.scol, A.sbase, A.soff,
+                   A.sperm, sval, x, z, y, theta, c, ig);
     };
     if (A.soff && A.sperm) go(sell_kernel<MODE, HAS_Z, true, true, T>);
     else if (A.soff) go(sell_kernel<MODE, HAS_Z, true, false, T>);

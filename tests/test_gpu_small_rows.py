@@ -57,3 +57,34 @@ def test_products_on_few_rows(solver, n, i, s):
                             beta=0.0, upper=True, n=n).cpu().numpy()
     ref = Z.T.astype(np.longdouble) @ X
     assert np.all(np.abs(T - ref) <= (s + 8) * u * (np.abs(Z.T) @ np.abs(X)))
+
+
+@pytest.mark.parametrize("n", [33, 4096, 4867, 20_000])
+def test_early_launches_keep_their_order(solver, n):
+    """A chain of short kernels that overwrite each other's inputs (columns
+    at odd 16-byte places, so that CTAs share cache lines) gives the same
+    bits every time, and the same as with a synchronisation after each."""
+    rng = np.random.default_rng(n)
+    i, s, ld = 21, 10, n + n % 2 + 2
+    solver.n = n
+    Q0, X0 = dev(rng.standard_normal((i, ld))), dev(rng.standard_normal((s, ld)))
+    Z = dev(np.ascontiguousarray(np.triu(rng.uniform(0.1, 0.2, (s, s))).T))
+
+    def chain(sync):
+        Q, X = Q0.clone(), X0.clone()
+        out = []
+        for _ in range(6):
+            for step in (lambda: out.append(solver.block_dot(Q, X)),
+                         lambda: solver.block_update(Q, out[-1] * (0.5 / n), X, n=n),
+                         lambda: out.append(solver.block_dot(X, X, sym=True)),
+                         lambda: solver.block_update(X, Z, Q[:s], alpha=1.0, beta=0.0, upper=True, n=n)):
+                step()
+                if sync:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return out + [Q, X]
+
+    ref = chain(True)
+    for _ in range(20):
+        for a, b in zip(chain(False), ref):
+            assert torch.equal(a, b)
