@@ -490,7 +490,8 @@ bool tc_forced() { return policy_now() == SG_TC_ALWAYS; }
 template <typename T>
 void block_dot_impl(int64_t n, const T* Q, int64_t ldq, int i, const T* X,
                     int64_t ldx, int s, double* W, int ldw, bool sym,
-                    double* part, int64_t part_cap, cudaStream_t st) {
+                    double* part, int64_t part_cap, cudaStream_t st, ColExps* eq = nullptr,
+                    ColExps* ex = nullptr) {
   if (i <= 0 || s <= 0) return;
   if (n <= 0) {
     for (int c = 0; c < s; ++c)
@@ -510,7 +511,7 @@ void block_dot_impl(int64_t n, const T* Q, int64_t ldq, int i, const T* X,
                "block_dot: workspace too small");
     int S = 0;
     oz_dot(n, reinterpret_cast<const double*>(Q), ldq, i, reinterpret_cast<const double*>(X),
-           ldx, s, reinterpret_cast<int*>(part + need), part, need, &S, st);
+           ldx, s, reinterpret_cast<int*>(part + need), part, need, &S, st, eq, ex);
     launch_reduce(i, s, S, part, W, ldw, false, st);
     return;
   }
@@ -962,9 +963,10 @@ int64_t block_dot_part_size(int64_t n, int i, int s) {
 
 void block_dot(int64_t n, const double* Q, int64_t ldq, int i,
                const double* X, int64_t ldx, int s, double* W, int ldw,
-               bool sym, double* part, int64_t part_cap, cudaStream_t st) {
+               bool sym, double* part, int64_t part_cap, cudaStream_t st, ColExps* eq,
+               ColExps* ex) {
   block_dot_impl<double>(n, Q, ldq, i, X, ldx, s, W, ldw, sym, part, part_cap,
-                         st);
+                         st, eq, ex);
 }
 
 void block_dot32(int64_t n, const float* Q, int64_t ldq, int i,
@@ -979,15 +981,16 @@ int64_t block_update_scratch(int i) { return (static_cast<int64_t>(i) + 1) / 2 +
 void block_update(int64_t n, const double* Q, int64_t ldq, int i,
                   const double* W, int ldw, double* X, int64_t ldx, int s,
                   double alpha, double beta, bool upper, double* scratch,
-                  int64_t scratch_doubles, cudaStream_t st) {
+                  int64_t scratch_doubles, cudaStream_t st, ColExps* eq, ColExps* ex) {
   if (n > 0 && i > 0 && s > 0 && scratch && scratch_doubles >= block_update_scratch(i) &&
       !tc_disabled() && oz_update_supported(n, Q, ldq, i, X, ldx, s) &&
       (tc_forced() || oz_update_pays(n, i, s, upper))) {
     // FP64 products on the tensor cores, exact digit slices
     oz_update(n, Q, ldq, i, W, ldw, X, ldx, s, alpha, beta, upper,
-              reinterpret_cast<int*>(scratch), st);
+              reinterpret_cast<int*>(scratch), st, eq, ex);
     return;
   }
+  if (ex) ex->valid = 0;
   block_update_impl<double>(n, Q, ldq, i, W, ldw, X, ldx, s, alpha, beta,
                             upper, st);
 }

@@ -675,6 +675,7 @@ constexpr uint32_t kUACol = 256;                        // A buffer b: 256 + 128
 // e_k, W' column exponents g_c
 struct OzUTables {
   alignas(16) uint32_t w[kUMaxK];
+  uint32_t top[kUN];               // largest finite |x|'s high word per output column
   int g[kUN];
 };
 
@@ -715,7 +716,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
 oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapX,
                  int64_t n, int i, int s, const double* __restrict__ W, int ldw,
                  double* __restrict__ X, int64_t ldx, double alpha, double beta, int upper,
-                 const int* __restrict__ eq, int* __restrict__ err) {
+                 const int* __restrict__ eq, int* __restrict__ eout, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char dsmem[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -780,7 +781,10 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   // relative to its column exponents g_c: B slices of every 64 columns of Q
   if (warp < kUWarps) {
     for (int k = tid; k < kUMaxK; k += kUSplit) tb.w[k] = near_word(k < i ? eq[k] : -4000);
-    if (tid < kUN) tb.g[tid] = -2147483647;
+    if (tid < kUN) {
+      tb.g[tid] = -2147483647;
+      tb.top[tid] = 0;
+    }
     uint4* z = reinterpret_cast<uint4*>(bsl);
     for (int e = tid; e < nkc * kUBChunk / 16; e += kUSplit) z[e] = make_uint4(0, 0, 0, 0);
   }
@@ -948,8 +952,15 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           } else {
             p = int96_to_double(hi, lo, gcol - 68) * alpha;
           }
-          if (r < n && c0 + cc < s)
-            xr[static_cast<int64_t>(cc) * ldx] = loadx ? fma(beta, xs[cc * kUM], p) : p;
+          if (loadx) p = fma(beta, xs[cc * kUM], p);
+          if (r < n && c0 + cc < s) xr[static_cast<int64_t>(cc) * ldx] = p;
+          if (eout) {
+            // the output column's exponent for the products that follow
+            uint32_t t = static_cast<uint32_t>(__double2hiint(p)) & 0x7FFFFFFFu;
+            if (r >= n || t >= 0x7FF00000u) t = 0;
+            t = __reduce_max_sync(0xffffffffu, t);
+            if (lane == 0) atomicMax(&tb.top[cg * kCols + cc], t);
+          }
           alo[cc] = lo0;
           ahi[cc] = hi0;
         }
@@ -1036,6 +1047,10 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (sh.fail && tid == 0) atomicExch(err, 1);
+  // (columns of zeros and subnormals keep the start value, as the cut takes
+  // both for zero)
+  if (eout && tid < kUN && n0 + tid < s && tb.top[tid] >= 0x00100000u)
+    atomicMax(eout + n0 + tid, static_cast<int>(tb.top[tid] >> 20) - 1022);
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
@@ -1115,6 +1130,21 @@ void col_exponents(int64_t n, const double* X, int64_t ld, int cols, int* e, cud
   col_exponent_kernel<<<dim3(cols, static_cast<unsigned>((n + rows - 1) / rows)), 256, 0, st>>>(
       n, X, ld, rows, e);
   SG_LAUNCH_CHECK();
+}
+
+// The exponents of a matrix's columns: those that the caller keeps, completed,
+// or all of them, in `scratch`.
+const int* exponents_of(int64_t n, const double* X, int64_t ld, int cols, ColExps* kept,
+                        int* scratch, cudaStream_t st) {
+  if (!kept) {
+    col_exponents(n, X, ld, cols, scratch, st);
+    return scratch;
+  }
+  if (kept->valid < cols) {
+    col_exponents(n, X + kept->valid * ld, ld, cols - kept->valid, kept->e + kept->valid, st);
+    kept->valid = cols;
+  }
+  return kept->e;
 }
 
 __device__ int g_oz_err;
@@ -1803,9 +1833,13 @@ bool oz_update_pays(int64_t n, int i, int s, bool upper) {
 
 void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, int ldw,
                double* X, int64_t ldx, int s, double alpha, double beta, bool upper, int* exps,
-               cudaStream_t st) {
+               cudaStream_t st, ColExps* eq, ColExps* ex) {
   int* err = oz_err_flag();
-  col_exponents(n, Q, ldq, i, exps, st);
+  const int* e = exponents_of(n, Q, ldq, i, eq, exps, st);
+  if (ex) {
+    SG_CUDA(cudaMemsetAsync(ex->e, 0x80, sizeof(int) * s, st));   // as col_exponents starts
+    ex->valid = s;
+  }
   CUtensorMap mq, mx;
   SG_REQUIRE(make_map64_box(&mq, Q, n, i, ldq) && make_map64_box(&mx, X, n, s, ldx), SG_ECUDA,
              "cuTensorMapEncodeTiled failed");
@@ -1814,7 +1848,7 @@ void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, 
   const int64_t ntiles = (n + kUM - 1) / kUM;
   const int64_t P = std::max<int64_t>(ct, std::min<int64_t>(device_sm_count(), ct * ntiles));
   oz_update_kernel<<<static_cast<unsigned>(P), kUThreads, oz_update_smem(i), st>>>(
-      mq, mx, n, i, s, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0, exps, err);
+      mq, mx, n, i, s, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0, e, ex ? ex->e : nullptr, err);
   SG_LAUNCH_CHECK();
   oz_check_error_pending.fetch_add(1);
 }
@@ -1832,18 +1866,15 @@ void oz_check_error(cudaStream_t st) {
 }
 
 void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int64_t ldx,
-            int s, int* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st) {
+            int s, int* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st,
+            ColExps* ceq, ColExps* cex) {
   int* err = oz_err_flag();
   int64_t rows = 0;
   const int64_t S = oz_splits(n, i, s, &rows);
   SG_REQUIRE(S * i * s <= part_cap, SG_EINVAL, "oz_dot: workspace too small");
-  int* eq = exps;
-  int* ex = exps + i;
-  col_exponents(n, Q, ldq, i, eq, st);
-  if (X == Q && s <= i)
-    SG_CUDA(cudaMemcpyAsync(ex, eq, sizeof(int) * s, cudaMemcpyDeviceToDevice, st));
-  else
-    col_exponents(n, X, ldx, s, ex, st);
+  const int* eq = exponents_of(n, Q, ldq, i, ceq, exps, st);
+  const int* ex = X == Q && ldx == ldq && s <= i ? eq
+                                                 : exponents_of(n, X, ldx, s, cex, exps + i, st);
   CUtensorMap mq, mx;
   SG_REQUIRE(make_map64(&mq, Q, n, i, ldq, kOM) && make_map64(&mx, X, n, s, ldx, kON), SG_ECUDA,
              "cuTensorMapEncodeTiled failed");

@@ -154,12 +154,23 @@ void axpy_f32_to_f64(int64_t n, double alpha, const float* d, double* x,
                      cudaStream_t st);
 void fill_zero(int64_t n, double* x, cudaStream_t st);
 
+// Exponents of the columns of an FP64 matrix (|x| < 2^e, as the tensor-core
+// products need them) that the caller keeps beside it: device ints e, of
+// which the first `valid` hold.  block_dot and block_update complete them
+// where they need them and set those of the columns that they write; whoever
+// else writes the columns sets valid to 0.
+struct ColExps {
+  int* e = nullptr;
+  int valid = 0;
+};
+
 // ------------------------------------------------------ dense kernels
 // W = Q^T X through split-n partials (workspace `part`, `part_cap`
 // doubles); sym: Q == X, only the upper tile triangle is computed.
 void block_dot(int64_t n, const double* Q, int64_t ldq, int i,
                const double* X, int64_t ldx, int s, double* W, int ldw,
-               bool sym, double* part, int64_t part_cap, cudaStream_t st);
+               bool sym, double* part, int64_t part_cap, cudaStream_t st,
+               ColExps* eq = nullptr, ColExps* ex = nullptr);
 void block_dot32(int64_t n, const float* Q, int64_t ldq, int i,
                  const float* X, int64_t ldx, int s, double* W, int ldw,
                  bool sym, double* part, int64_t part_cap, cudaStream_t st);
@@ -176,7 +187,8 @@ void block_dot_capped(int64_t n, const double* Q, int64_t ldq, int i,
 void block_update(int64_t n, const double* Q, int64_t ldq, int i,
                   const double* W, int ldw, double* X, int64_t ldx, int s,
                   double alpha, double beta, bool upper, double* scratch,
-                  int64_t scratch_doubles, cudaStream_t st);
+                  int64_t scratch_doubles, cudaStream_t st, ColExps* eq = nullptr,
+                  ColExps* ex = nullptr);
 int64_t block_update_scratch(int i);
 
 // process-wide tensor-core policy of the FP64 block products (SG_TC_*);
@@ -217,9 +229,11 @@ bool oz_update_supported(int64_t n, const double* Q, int64_t ldq, int i, const d
 bool oz_update_pays(int64_t n, int i, int s, bool upper);
 void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, int ldw,
                double* X, int64_t ldx, int s, double alpha, double beta, bool upper, int* exps,
-               cudaStream_t st);
+               cudaStream_t st,
+               ColExps* eq, ColExps* ex);
 void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int64_t ldx,
-            int s, int* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st);
+            int s, int* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st,
+            ColExps* eq, ColExps* ex);
 void oz_check_error(cudaStream_t st);
 // Tensor-core FP32 Gram G = X^T X (s <= 128 columns) from exact digit
 // slices: split partials of the upper triangle (entry (m, n), m <= n, at

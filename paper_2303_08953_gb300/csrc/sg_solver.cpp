@@ -34,7 +34,7 @@ void dev_alloc(T** p, size_t count) {
 
 // Small-matrix slots inside h->small / h->hbuf (offsets in doubles).
 struct Slots {
-  int64_t W, G, Z, Y, scal, H, wn, total;
+  int64_t W, G, Z, Y, scal, H, wn, E, total;
 };
 Slots slots_for(int m, int k) {
   Slots s{};
@@ -47,6 +47,7 @@ Slots slots_for(int m, int k) {
   s.scal = o; o += 16;        // scalars (norms)
   s.H = o;    o += kk * kk;   // Arnoldi pre-pass Hessenberg ((k+1) x k)
   s.wn = o;   o += kk;        // pre-pass norms before projection
+  s.E = o;    o += (mm + 2 * kk + 1) / 2;   // column exponents (ints): Q, V, Y
   s.total = o;
   return s;
 }
@@ -164,15 +165,13 @@ template <> struct Basis<double> {
   }
   static void bdot(int64_t n, const double* Q, int64_t ldq, int i, const double* X,
                    int64_t ldx, int s, double* W, int ldw, bool sym, double* part,
-                   int64_t cap, cudaStream_t st) {
-    block_dot(n, Q, ldq, i, X, ldx, s, W, ldw, sym, part, cap, st);
+                   int64_t cap, cudaStream_t st, ColExps* eq, ColExps* ex) {
+    block_dot(n, Q, ldq, i, X, ldx, s, W, ldw, sym, part, cap, st, eq, ex);
   }
   static void bupd(sg_handle* h, int64_t n, const double* Q, int64_t ldq, int i,
                    const double* W, int ldw, double* X, int64_t ldx, int s, double al,
-                   double be, bool up, cudaStream_t st) {
-    // Q's column exponents of the tensor-core form go to the (then idle)
-    // split-partials buffer
-    block_update(n, Q, ldq, i, W, ldw, X, ldx, s, al, be, up, h->part, h->part_cap, st);
+                   double be, bool up, cudaStream_t st, ColExps* eq, ColExps* ex) {
+    block_update(n, Q, ldq, i, W, ldw, X, ldx, s, al, be, up, h->part, h->part_cap, st, eq, ex);
   }
   static void gemv(int64_t n, int k, const double* Q, int64_t ldq, const double* y,
                    double* x, cudaStream_t st) {
@@ -194,14 +193,14 @@ template <> struct Basis<float> {
   }
   static void bdot(int64_t n, const float* Q, int64_t ldq, int i, const float* X,
                    int64_t ldx, int s, double* W, int ldw, bool sym, double* part,
-                   int64_t cap, cudaStream_t st) {
+                   int64_t cap, cudaStream_t st, ColExps*, ColExps*) {
     block_dot32(n, Q, ldq, i, X, ldx, s, W, ldw, sym, part, cap, st);
   }
   // the tensor-core update stages W's TF32 split in the (then idle)
   // split-partials buffer of the workspace
   static void bupd(sg_handle* h, int64_t n, const float* Q, int64_t ldq, int i,
                    const double* W, int ldw, float* X, int64_t ldx, int s, double al,
-                   double be, bool up, cudaStream_t st) {
+                   double be, bool up, cudaStream_t st, ColExps*, ColExps*) {
     block_update32(n, Q, ldq, i, W, ldw, X, ldx, s, al, be, up, h->part, h->part_cap, st);
   }
   static void gemv(int64_t n, int k, const float* Q, int64_t ldq, const double* y,
@@ -419,6 +418,12 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
   double* yd = h->small + sl.Y;
   double* sc = h->small + sl.scal;
   double* hb = h->hbuf;
+  // The column exponents of Q, the block V and the block Y (FP64 basis): a
+  // column of Q keeps its own through the cycle and the updates give those of
+  // what they write, so that only the powers are read for them (reading every
+  // operand of every product took 8 % of the 128^3 FP64 solve).
+  int* exps = reinterpret_cast<int*>(h->small + sl.E);
+  ColExps eQ{exps, 0}, eX{exps + h->ws_m + 1, 0}, eY{exps + h->ws_m + h->ws_k + 2, 0};
   const int max_iters = o.max_iters > 0 ? o.max_iters : 50 * m;
 
   auto device_norm = [&](const double* v, double* slot) {
@@ -456,6 +461,7 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
   for (;;) {
     // Q_1 = r / beta
     B::from_f64(n, h->rvec, Qb, 1.0 / beta, st);
+    eQ.valid = 0;
     if (!have_shifts) {
       const double tp = now_ms();
       int steps = 0;
@@ -504,10 +510,11 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
       }
       SG_CUDA(cudaEventRecord(h->ev[1], st));
       T* X = Vb + ld;
+      eX.valid = 0;
       // first BCGS: W = Q^T X; X -= Q W; G = X^T X
-      B::bdot(n, Qb, ld, i, X, ld, s_eff, Wd, i, false, h->part, h->part_cap, st);
-      B::bupd(h, n, Qb, ld, i, Wd, i, X, ld, s_eff, -1.0, 1.0, false, st);
-      B::bdot(n, X, ld, s_eff, X, ld, s_eff, Gd, s_eff, true, h->part, h->part_cap, st);
+      B::bdot(n, Qb, ld, i, X, ld, s_eff, Wd, i, false, h->part, h->part_cap, st, &eQ, &eX);
+      B::bupd(h, n, Qb, ld, i, Wd, i, X, ld, s_eff, -1.0, 1.0, false, st, &eQ, &eX);
+      B::bdot(n, X, ld, s_eff, X, ld, s_eff, Gd, s_eff, true, h->part, h->part_cap, st, &eX, &eX);
       fetch(Wd, static_cast<int64_t>(i) * s_eff, hb);
       fetch(Gd, static_cast<int64_t>(s_eff) * s_eff, hb + static_cast<int64_t>(i) * s_eff);
       SG_CUDA(cudaEventRecord(h->ev[2], st));
@@ -551,14 +558,15 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
         SG_CUDA(cudaMemcpyAsync(Zd, hb + sl.Z, sizeof(double) * p1 * p1, cudaMemcpyHostToDevice, st));
         SG_CUDA(cudaEventRecord(h->ev[1], st));
         // Q_k = X(:, 1:p) Z^-1, then second BCGS and the second Gram
-        B::bupd(h, n, X, ld, p1, Zd, p1, Yb, ld, p1, 1.0, 0.0, true, st);
-        B::bdot(n, Qb, ld, i, Yb, ld, p1, Wd, i, false, h->part, h->part_cap, st);
-        B::bupd(h, n, Qb, ld, i, Wd, i, Yb, ld, p1, -1.0, 1.0, false, st);
+        B::bupd(h, n, X, ld, p1, Zd, p1, Yb, ld, p1, 1.0, 0.0, true, st, &eX, &eY);
+        B::bdot(n, Qb, ld, i, Yb, ld, p1, Wd, i, false, h->part, h->part_cap, st, &eQ, &eY);
+        B::bupd(h, n, Qb, ld, i, Wd, i, Yb, ld, p1, -1.0, 1.0, false, st, &eQ, &eY);
         // Gram of the block the first pass already orthonormalised: FP64
         // uses the symmetric kernel; the FP32 basis needs only FP32-level
         // accuracy here (its condition number is ~1), so it goes to the
         // tensor-core kernel like the projections
-        B::bdot(n, Yb, ld, p1, Yb, ld, p1, Gd, p1, sizeof(T) == 8, h->part, h->part_cap, st);
+        B::bdot(n, Yb, ld, p1, Yb, ld, p1, Gd, p1, sizeof(T) == 8, h->part, h->part_cap, st,
+                &eY, &eY);
         fetch(Wd, static_cast<int64_t>(i) * p1, hb);
         fetch(Gd, static_cast<int64_t>(p1) * p1, hb + static_cast<int64_t>(i) * p1);
         SG_CUDA(cudaEventRecord(h->ev[2], st));
@@ -597,8 +605,10 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
           log.t_host += now_ms() - th1;
           SG_CUDA(cudaMemcpyAsync(Zd, hb + sl.Z, sizeof(double) * q * q, cudaMemcpyHostToDevice, st));
           // Q_k = Q_k(:, 1:q) Z~^-1 into Q's next columns
+          ColExps eN{eQ.e + i, 0};
           B::bupd(h, n, Yb, ld, q, Zd, q, Qb + static_cast<int64_t>(i) * ld, ld, q,
-                  1.0, 0.0, true, st);
+                  1.0, 0.0, true, st, &eY, &eN);
+          if (eQ.valid == i) eQ.valid = i + eN.valid;
         }
       }
       const double th2 = now_ms();

@@ -115,3 +115,29 @@ def test_block_update_hard_digits(solver, tc_always, n, alpha, beta):
             sub = abs(Fraction(alpha)) * sum(abs(Fraction(Wm[k, c])) for k in range(i)) * Fraction(2) ** -1022
             tol = drop + sub + 4 * (abs(p) + abs(ref)) / 2 ** 53
             assert abs(Fraction(got[c, r]) - ref) <= tol, (r, c)
+
+
+@pytest.mark.parametrize("m,s", [(30, 7), (24, 24), (17, 5)])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -40, 2.0 ** 40])
+def test_solve_with_kept_exponents(tc_always, m, s, scale):
+    """Whole restarted solves whose block products all take their column
+    exponents from the updates that wrote the columns: the solution of
+    A x = scale b (residual to 1e-12; the system's condition number is
+    below 1e3) within 1e-9 of the FP64 direct one."""
+    import scipy.sparse as sp
+    import scipy.sparse.linalg as spl
+
+    import workloads as W
+    A = W.config_c1(32)["A"]
+    M = sp.csr_matrix((A.val, A.colind, A.rowptr), shape=(A.n, A.n))
+    rng = np.random.default_rng(m)
+    b = rng.standard_normal(A.n) * scale
+    solver = sg.Solver(0)
+    try:
+        solver.analyze_csr(A)
+        x, info = solver.solve(dev(b), m=m, s=s, tol=1e-12)
+        assert info.converged and info.restarts >= 1
+        ref = spl.spsolve(M.tocsc(), b)
+        assert np.linalg.norm(x.cpu().numpy() - ref) <= 1e-9 * np.linalg.norm(ref)
+    finally:
+        solver.close()
