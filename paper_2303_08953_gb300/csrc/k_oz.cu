@@ -1853,16 +1853,24 @@ void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, 
   oz_check_error_pending.fetch_add(1);
 }
 
-void oz_check_error(cudaStream_t st) {
+void oz_fetch_error(int* host, cudaStream_t st) {
+  *host = 0;
   if (oz_check_error_pending.exchange(0) == 0) return;
-  int* f = oz_err_flag();
+  SG_CUDA(cudaMemcpyAsync(host, oz_err_flag(), sizeof(int), cudaMemcpyDeviceToHost, st));
+}
+
+void oz_report_error(int host, cudaStream_t st) {
+  if (!host) return;
+  SG_CUDA(cudaMemsetAsync(oz_err_flag(), 0, sizeof(int), st));
+  throw Error(SG_ECUDA, "tensor-core FP64 block dot: a bounded wait ran out");
+}
+
+void oz_check_error(cudaStream_t st) {
+  if (oz_check_error_pending.load() == 0) return;
   int host = 0;
-  SG_CUDA(cudaMemcpyAsync(&host, f, sizeof(int), cudaMemcpyDeviceToHost, st));
+  oz_fetch_error(&host, st);
   SG_CUDA(cudaStreamSynchronize(st));
-  if (host) {
-    SG_CUDA(cudaMemsetAsync(f, 0, sizeof(int), st));
-    throw Error(SG_ECUDA, "tensor-core FP64 block dot: a bounded wait ran out");
-  }
+  oz_report_error(host, st);
 }
 
 void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int64_t ldx,

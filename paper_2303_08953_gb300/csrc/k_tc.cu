@@ -402,16 +402,24 @@ int* tc_err_flag() {
   return ptr[dev];
 }
 
-void tc_check_error(cudaStream_t st) {
+void tc_fetch_error(int* host, cudaStream_t st) {
+  *host = 0;
   if (tc_check_error_pending.exchange(0) == 0) return;
-  int* f = tc_err_flag();
+  SG_CUDA(cudaMemcpyAsync(host, tc_err_flag(), sizeof(int), cudaMemcpyDeviceToHost, st));
+}
+
+void tc_report_error(int host, cudaStream_t st) {
+  if (!host) return;
+  SG_CUDA(cudaMemsetAsync(tc_err_flag(), 0, sizeof(int), st));
+  throw Error(SG_ECUDA, "tensor-core block dot: a bounded wait ran out");
+}
+
+void tc_check_error(cudaStream_t st) {
+  if (tc_check_error_pending.load() == 0) return;
   int host = 0;
-  SG_CUDA(cudaMemcpyAsync(&host, f, sizeof(int), cudaMemcpyDeviceToHost, st));
+  tc_fetch_error(&host, st);
   SG_CUDA(cudaStreamSynchronize(st));
-  if (host) {
-    SG_CUDA(cudaMemsetAsync(f, 0, sizeof(int), st));
-    throw Error(SG_ECUDA, "tensor-core block dot: a bounded wait ran out");
-  }
+  tc_report_error(host, st);
 }
 
 void tc_dot(int64_t n, const float* Q, int64_t ldq, int i, const float* X, int64_t ldx,

@@ -450,16 +450,24 @@ void tc_update(int64_t n, const float* Q, int64_t ldq, int i, const double* W, i
   SG_LAUNCH_CHECK();
 }
 
-void tc_update_check_error(cudaStream_t st) {
+void tc_update_fetch_error(int* host, cudaStream_t st) {
+  *host = 0;
   if (tc_update_check_error_pending.exchange(0) == 0) return;
-  int* f = err_flag();
+  SG_CUDA(cudaMemcpyAsync(host, err_flag(), sizeof(int), cudaMemcpyDeviceToHost, st));
+}
+
+void tc_update_report_error(int host, cudaStream_t st) {
+  if (!host) return;
+  SG_CUDA(cudaMemsetAsync(err_flag(), 0, sizeof(int), st));
+  throw Error(SG_ECUDA, "tensor-core block update: a bounded wait ran out");
+}
+
+void tc_update_check_error(cudaStream_t st) {
+  if (tc_update_check_error_pending.load() == 0) return;
   int host = 0;
-  SG_CUDA(cudaMemcpyAsync(&host, f, sizeof(int), cudaMemcpyDeviceToHost, st));
+  tc_update_fetch_error(&host, st);
   SG_CUDA(cudaStreamSynchronize(st));
-  if (host) {
-    SG_CUDA(cudaMemsetAsync(f, 0, sizeof(int), st));
-    throw Error(SG_ECUDA, "tensor-core block update: a bounded wait ran out");
-  }
+  tc_update_report_error(host, st);
 }
 
 }  // namespace sg

@@ -212,6 +212,12 @@ void tc_dot(int64_t n, const float* Q, int64_t ldq, int i, const float* X,
             int64_t ldx, int s, double* part, int64_t part_cap, int* nsplit,
             cudaStream_t st);
 void tc_check_error(cudaStream_t st);
+// The same in two halves, for a caller that synchronises anyway: fetch_error
+// queues the flag's copy to `host` (pinned; set to 0 at once where no kernel
+// has run since the last check), report_error, after the synchronisation,
+// throws on a flag that was set.
+void tc_fetch_error(int* host, cudaStream_t st);
+void tc_report_error(int host, cudaStream_t st);
 // Tensor-core (tcgen05, TMA) FP64 block dot W = Q^T X from exact 8-bit
 // digit slices of both operands: split partials into `part` (part_cap
 // doubles), column exponents into `exps` (oz_exp_ints(i, s) ints), number of
@@ -235,6 +241,8 @@ void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int
             int s, int* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st,
             ColExps* eq, ColExps* ex);
 void oz_check_error(cudaStream_t st);
+void oz_fetch_error(int* host, cudaStream_t st);
+void oz_report_error(int host, cudaStream_t st);
 // Tensor-core FP32 Gram G = X^T X (s <= 128 columns) from exact digit
 // slices: split partials of the upper triangle (entry (m, n), m <= n, at
 // m + n s) into `part`, column exponents into `exps` (s ints); a bounded
@@ -253,6 +261,8 @@ void tc_update(int64_t n, const float* Q, int64_t ldq, int i, const double* W,
                bool upper, float* scratch, int64_t scratch_floats,
                cudaStream_t st);
 void tc_update_check_error(cudaStream_t st);
+void tc_update_fetch_error(int* host, cudaStream_t st);
+void tc_update_report_error(int host, cudaStream_t st);
 
 // dst[k] = src[idx[k]], k < count (device arrays).
 // Structure checks of a square CSR matrix on the device (synchronises):

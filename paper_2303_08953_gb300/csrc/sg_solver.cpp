@@ -434,6 +434,25 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
     SG_CUDA(cudaMemcpyAsync(dst, src, sizeof(double) * count, cudaMemcpyDeviceToHost, st));
   };
 
+  // The tensor-core kernels' timeout flags come back with the block's sums,
+  // under the one synchronisation: copies of their own, each with its own
+  // synchronisation, took about 15 us apiece, up to six of them a block.
+  int* flags = reinterpret_cast<int*>(hb + sl.E);
+  auto fetch_errors = [&] {
+    oz_fetch_error(flags, st);
+    if (sizeof(T) == 4) {
+      tc_fetch_error(flags + 1, st);
+      tc_update_fetch_error(flags + 2, st);
+    }
+  };
+  auto report_errors = [&] {
+    oz_report_error(flags[0], st);
+    if (sizeof(T) == 4) {
+      tc_report_error(flags[1], st);
+      tc_update_report_error(flags[2], st);
+    }
+  };
+
   // r = b - A x0, beta0 (Alg. 4, first line)
   residual(M, h->bvec, h->xvec, h->rvec, st);
   device_norm(h->rvec, sc);
@@ -518,9 +537,9 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
       fetch(Wd, static_cast<int64_t>(i) * s_eff, hb);
       fetch(Gd, static_cast<int64_t>(s_eff) * s_eff, hb + static_cast<int64_t>(i) * s_eff);
       SG_CUDA(cudaEventRecord(h->ev[2], st));
+      fetch_errors();
       SG_CUDA(cudaStreamSynchronize(st));
-      if (sizeof(T) == 4) { tc_check_error(st); tc_update_check_error(st); oz_check_error(st); }
-      else oz_check_error(st);
+      report_errors();
       {
         float a = 0, b = 0;
         cudaEventElapsedTime(&a, h->ev[0], h->ev[1]);
@@ -570,9 +589,9 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
         fetch(Wd, static_cast<int64_t>(i) * p1, hb);
         fetch(Gd, static_cast<int64_t>(p1) * p1, hb + static_cast<int64_t>(i) * p1);
         SG_CUDA(cudaEventRecord(h->ev[2], st));
+        fetch_errors();
         SG_CUDA(cudaStreamSynchronize(st));
-        if (sizeof(T) == 4) { tc_check_error(st); tc_update_check_error(st); oz_check_error(st); }
-        else oz_check_error(st);
+        report_errors();
         {
           float b = 0;
           cudaEventElapsedTime(&b, h->ev[1], h->ev[2]);
