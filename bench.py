@@ -234,13 +234,6 @@ def mgs_bytes(A, k):
     return sum(8 * A.n * (j + 3) for j in range(k))
 
 
-# DRAM bytes of one MGS launch per row and per vector it streams (j + 2
-# vectors read at step j), from the ncu capture of step j = 58 at
-# 2,097,152 rows: 1,007,194,000 + 3,276,544 bytes over 60 vectors
-# (profiles/arnoldi_mgs_resident_fp64_randband_2M_j58.md).
-MGS_DRAM_BYTES_PER_ROW_VECTOR = (1_006_732_000 + 3_225_344) / 2_097_152 / 60
-
-
 # ------------------------------------------------------------ CPU oracle
 # The oracle's complete solve of the headline workload takes minutes on the
 # host (it is plain numpy, one projection at a time), so the CPU baseline is
@@ -409,28 +402,25 @@ def run_ours(args):
     t_launch = (t_pre - PREPASS_STEPS * t_sp) / PREPASS_STEPS
     fl = mgs_flops(A, PREPASS_STEPS) / PREPASS_STEPS
     by = mgs_bytes(A, PREPASS_STEPS) / PREPASS_STEPS
-    vec = sum(j + 2 for j in range(PREPASS_STEPS)) / PREPASS_STEPS
     pk = measured_peaks()
     hbm = pk["hbm_gbs"] if pk else 6800.0
     hbm_src = "MEASURED_PEAKS.json hbm_gbs" if pk else "fallback"
-    ach = fl / t_launch / 1e12
+    # fixed point: integer multiply-adds in place of the FP64 flops counted
+    # here, so the stream of the basis is the roofline left to report against
+    mgs_gbs = by / t_launch / 1e9
     out["roofline"] = {
-        "kernel": f"arnoldi_mgs_resident_kernel FP64 (MGS phases of one Ritz pre-pass step, "
-                  f"w in shared memory; mean of the {PREPASS_STEPS} launches of one pre-pass)",
-        "bound": "alu", "achieved": round(ach, 4),
-        "peak": round(FP64_ALU_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
-        "frac": round(ach / FP64_ALU_PEAK_TFLOPS, 4),
-        "traffic": int(round(MGS_DRAM_BYTES_PER_ROW_VECTOR * n * vec)),
-        "traffic_source": "ncu dram__bytes_read+write of the launch at step j = 58, 2,097,152 "
-                          "rows, per row and streamed vector, scaled to this n and the mean "
-                          "step (profiles/arnoldi_mgs_resident_fp64_randband_2M_j58.md)",
+        "kernel": f"arnoldi_mgs_resident_kernel FP64 basis in fixed point (MGS phases of one Ritz "
+                  f"pre-pass step, w in shared memory; mean of the {PREPASS_STEPS} launches of "
+                  f"one pre-pass)",
+        "bound": "hbm", "achieved": round(mgs_gbs, 1), "peak": hbm, "unit": "GB/s",
+        "frac": round(mgs_gbs / hbm, 4), "traffic": None,
         "launch_ms": round(t_launch * 1e3, 4),
         "prepass_ms": round(t_pre * 1e3, 2),
         "algorithmic_flops_per_launch": int(fl),
         "algorithmic_bytes_per_launch": int(by),
-        "hbm_frac": round(by / t_launch / 1e9 / hbm, 4),
-        "peak_source": "derived: 152 SMs x 2.07 GHz x 4 FP64 flop/clk/SM "
-                       "(nominal 1.25 TFLOP/s FP64)"}
+        "fp64_equivalent_tflops": round(fl / t_launch / 1e12, 4),
+        "fp64_pipe_peak_tflops": round(FP64_ALU_PEAK_TFLOPS, 4),
+        "peak_source": hbm_src}
 
     # secondary: the MPK's SpMV against HBM (timed above)
     gbs = spmv_bytes(A) / t_sp / 1e9
