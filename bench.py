@@ -234,6 +234,13 @@ def mgs_bytes(A, k):
     return sum(8 * A.n * (j + 3) for j in range(k))
 
 
+# DRAM bytes of one MGS launch per row and per vector it streams (j + 2
+# vectors read at step j), from the ncu capture of step j = 58 at
+# 2,097,152 rows: 1,006,831,000 + 3,212,800 bytes over 60 vectors
+# (profiles/arnoldi_mgs_resident_fp64_randband_2M_j58.md).
+MGS_DRAM_BYTES_PER_ROW_VECTOR = (1_006_831_000 + 3_212_800) / 2_097_152 / 60
+
+
 # ------------------------------------------------------------ CPU oracle
 # The oracle's complete solve of the headline workload takes minutes on the
 # host (it is plain numpy, one projection at a time), so the CPU baseline is
@@ -402,6 +409,7 @@ def run_ours(args):
     t_launch = (t_pre - PREPASS_STEPS * t_sp) / PREPASS_STEPS
     fl = mgs_flops(A, PREPASS_STEPS) / PREPASS_STEPS
     by = mgs_bytes(A, PREPASS_STEPS) / PREPASS_STEPS
+    vec = sum(j + 2 for j in range(PREPASS_STEPS)) / PREPASS_STEPS
     pk = measured_peaks()
     hbm = pk["hbm_gbs"] if pk else 6800.0
     hbm_src = "MEASURED_PEAKS.json hbm_gbs" if pk else "fallback"
@@ -413,7 +421,11 @@ def run_ours(args):
                   f"pre-pass step, w in shared memory; mean of the {PREPASS_STEPS} launches of "
                   f"one pre-pass)",
         "bound": "hbm", "achieved": round(mgs_gbs, 1), "peak": hbm, "unit": "GB/s",
-        "frac": round(mgs_gbs / hbm, 4), "traffic": None,
+        "frac": round(mgs_gbs / hbm, 4),
+        "traffic": int(round(MGS_DRAM_BYTES_PER_ROW_VECTOR * n * vec)),
+        "traffic_source": "ncu dram__bytes_read+write of the launch at step j = 58, 2,097,152 "
+                          "rows, per row and streamed vector, scaled to this n and the mean "
+                          "step (profiles/arnoldi_mgs_resident_fp64_randband_2M_j58.md)",
         "launch_ms": round(t_launch * 1e3, 4),
         "prepass_ms": round(t_pre * 1e3, 2),
         "algorithmic_flops_per_launch": int(fl),

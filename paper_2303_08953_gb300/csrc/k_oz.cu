@@ -636,7 +636,7 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
 // relative to W' column c's exponent g_c, every product of the sum carries
 // the one weight 2^(g_c - 124), so the level sums are exact as above.  The
 // digits are FP16 numbers here (integers of at most 8 bits are exact in
-// either 16-bit type; FP16's wider mantissa lets one packed subtraction
+// either 16-bit type; FP16's wider mantissa lets one packed FMA
 // turn two digit bytes into two FP16 digits).
 // Tile: 128 rows (MMA M, tensor-memory lanes) x 32 columns of X (MMA N);
 // one CTA per SM walks the row tiles of one column tile in stages of 32
