@@ -405,6 +405,7 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
+    __syncwarp();   // .aligned, after a branch of one thread
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&sh.tmem_base)),
                  "r"(kOTmemCols)
@@ -771,6 +772,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
+    __syncwarp();   // .aligned, after a branch of one thread
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&sh.tmem_base)),
                  "r"(kOTmemCols)
@@ -1052,6 +1054,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   if (eout && tid < kUN && n0 + tid < s && tb.top[tid] >= 0x00100000u)
     atomicMax(eout + n0 + tid, static_cast<int>(tb.top[tid] >> 20) - 1022);
   if (warp == 0) {
+    __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(kOTmemCols)
@@ -1398,6 +1401,7 @@ oz_gram32_kernel(const __grid_constant__ CUtensorMap mapX, int64_t n, int s,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
+    __syncwarp();   // .aligned, after a branch of one thread
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&sh.tmem_base)),
                  "r"(kOTmemCols)

@@ -607,8 +607,11 @@ __device__ __forceinline__ long long fx_scale(long long x, int nh, int nl) {
 }
 
 // Tensor memory as storage: this thread's lane, four pairs of rows in 16
-// consecutive columns.
+// consecutive columns.  These instructions are .aligned: the whole warp has
+// to execute them converged, and their callers branch per lane at the ragged
+// end of a CTA's rows, so each of the three converges the warp itself.
 __device__ __forceinline__ void fx_tmem_st(uint32_t addr, const int4* v) {
+  __syncwarp();
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
       "%14,%15,%16};" ::"r"(addr),
@@ -620,6 +623,7 @@ __device__ __forceinline__ void fx_tmem_st(uint32_t addr, const int4* v) {
 // (the wait is in the same statement: no use of the registers can move
 // before it)
 __device__ __forceinline__ void fx_tmem_ld(uint32_t addr, int4* v) {
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
       "%15}, [%16];\n\t"
@@ -629,6 +633,10 @@ __device__ __forceinline__ void fx_tmem_ld(uint32_t addr, int4* v) {
         "=r"(v[3].x), "=r"(v[3].y), "=r"(v[3].z), "=r"(v[3].w)
       : "r"(addr)
       : "memory");
+}
+__device__ __forceinline__ void fx_tmem_wait_st() {
+  __syncwarp();
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 // T 2^s; rounded to the nearest integer for s < 0
@@ -977,12 +985,11 @@ arnoldi_mgs_resident_kernel(int n, int rows_cta, double* V, int64_t ld, int j, d
           }
         }
         if (k < kFxTmem) {
-          __syncwarp();
           fx_tmem_st(tm + 32 * k, a);
           fx_tmem_st(tm + 32 * k + 16, b);
         }
       }
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      fx_tmem_wait_st();
       warp_sums(h0, c, 0);
       warp_sums(h1, d, 1);
     }
@@ -1075,10 +1082,7 @@ arnoldi_mgs_resident_kernel(int n, int rows_cta, double* V, int64_t ld, int j, d
         }
         if (k < kFxTmem) fx_tmem_st(tq + 32 * k, y);
       }
-      if (nb < nbt && nb < kFxTmem) {
-        __syncwarp();
-        fx_tmem_ld(tq + 32 * nb, a);
-      }
+      if (nb < nbt && nb < kFxTmem) fx_tmem_ld(tq + 32 * nb, a);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int p = tail + u * T + t;
@@ -1092,9 +1096,8 @@ arnoldi_mgs_resident_kernel(int n, int rows_cta, double* V, int64_t ld, int j, d
           fx_flush(hh, c);
         }
       }
-      __syncwarp();
       if (nb < nbt && nb < kFxTmem) fx_tmem_st(tq + 32 * nb, v);
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      fx_tmem_wait_st();
       if (q + 3 <= j) load_first(q + 1);
       warp_sums(hh, c, b);
       if (warp == 1) {
@@ -1152,7 +1155,6 @@ arnoldi_mgs_resident_kernel(int n, int rows_cta, double* V, int64_t ld, int j, d
       for (int k = 0; k < nbt; ++k) {
         int4 x[U], y[U];
         if (k < kFxTmem) {
-          __syncwarp();
           fx_tmem_ld(tm + 32 * k + 16 * ((j + 1) & 1), x);
           fx_tmem_ld(tm + 32 * k + 16 * (j & 1), y);
         } else {

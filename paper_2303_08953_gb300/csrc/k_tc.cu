@@ -112,6 +112,7 @@ tc_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
+    __syncwarp();   // .aligned, after a branch of one thread
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&sh.tmem_base)),
                  "r"(kTmemCols)
@@ -270,6 +271,7 @@ tc_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
     for (int c0 = 0; c0 < BN; c0 += 16) {
       uint32_t v[16];
       const uint32_t taddr = tmem + (static_cast<uint32_t>(warp * 32) << 16) + c0;
+      __syncwarp();   // .aligned, after the stores of the rows inside M
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
           : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),

@@ -112,6 +112,7 @@ tc_update_kernel(const __grid_constant__ CUtensorMap mapQ,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
+    __syncwarp();   // .aligned, after a branch of one thread
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&sh.tmem_base)),
                  "r"(kTmemCols)
@@ -273,6 +274,7 @@ tc_update_kernel(const __grid_constant__ CUtensorMap mapQ,
       named_sync(1, 128);
       if (*reinterpret_cast<volatile int*>(&sh.epi_stop)) break;
       if (tid == 0) x_pending = false;
+      __syncwarp();   // the loads below are .aligned
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       for (int c0 = 0; c0 < BN; c0 += 16) {
         uint32_t v[16];
