@@ -45,8 +45,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // (whole warps idle on padded rows, otherwise on padded columns).
 template <int BM, int BN, int TM, int TN, bool MW, bool EXACT, typename T>
 __global__ void __launch_bounds__(kThreads)
-dot_tile_kernel(int64_t K, int M, int N, const T* __restrict__ A,
-                int64_t lda, const T* __restrict__ B, int64_t ldb,
+dot_tile_kernel(int64_t K, int M, int N, const T* A, int64_t lda, const T* B, int64_t ldb,
                 double* __restrict__ part, int64_t rows_per_split, int sym) {
   constexpr bool kF32 = sizeof(T) == 4;
   constexpr int TMN = BM / TM, TNN = BN / TN;
@@ -164,8 +163,8 @@ constexpr int kSmallOut = 256;
 constexpr int kSmallCols = 160;   // M + N: the staged rows fit 48 KB of shared memory
 
 __global__ void __launch_bounds__(kSmallOut)
-dot_small_kernel(int64_t K, int M, int N, const double* __restrict__ A, int64_t lda,
-                 const double* __restrict__ B, int64_t ldb, double* __restrict__ part,
+dot_small_kernel(int64_t K, int M, int N, const double* A, int64_t lda,
+                 const double* B, int64_t ldb, double* __restrict__ part,
                  int64_t rows_per_split, int sym) {
   wait_previous();
   release_next();
@@ -215,8 +214,7 @@ dot_small_kernel(int64_t K, int M, int N, const double* __restrict__ A, int64_t 
 // (m, n) and (n, m).  One warp per output: lane l adds splits l, l+32, ...
 // in order, then a fixed xor-shuffle tree combines the lanes, so the
 // result is deterministic and the S loads are issued 32 at a time.
-__global__ void reduce_parts_kernel(int M, int N, int S,
-                                    const double* __restrict__ part,
+__global__ void reduce_parts_kernel(int M, int N, int S, const double* part,
                                     double* __restrict__ W, int ldw, int sym) {
   wait_previous();
   release_next();
@@ -669,8 +667,8 @@ update_wide_kernel(int64_t K, int M, int N, const float* __restrict__ A, int64_t
 
 template <int UR, int UN, int TR, int TN, typename T>
 __global__ void __launch_bounds__(kThreads)
-update_kernel(int64_t K, int M, int N, const T* __restrict__ A, int64_t lda,
-              const double* __restrict__ B, int ldb, T* __restrict__ C,
+update_kernel(int64_t K, int M, int N, const T* A, int64_t lda,
+              const double* B, int ldb, T* __restrict__ C,
               int64_t ldc, double alpha, double beta, int upper) {
   wait_previous();
   release_next();
@@ -753,8 +751,8 @@ constexpr int kThinPass = 8;
 
 template <int MAXI, int MODE, typename T>
 __global__ void __launch_bounds__(kThreads)
-update_thin_kernel(int64_t n, int i, int s, const T* __restrict__ Q, int64_t ldq,
-                   const double* __restrict__ W, int ldw, T* __restrict__ X, int64_t ldx,
+update_thin_kernel(int64_t n, int i, int s, const T* Q, int64_t ldq,
+                   const double* W, int ldw, T* __restrict__ X, int64_t ldx,
                    double alpha, double beta, int upper) {
   wait_previous();
   release_next();

@@ -12,8 +12,8 @@
 // sptr[q] + 32 j + l, padded to the slice's longest row with column -1.
 // Lane l of a warp then walks row 32q + l while the warp reads each entry
 // index j as one coalesced 256-byte (values) and 128-byte (indices) line,
-// with no staging and no barriers; x is gathered through the read-only
-// path (stencil locality gives cache hits).  Up to eight entries per row
+// with no staging and no barriers; x is gathered through L1 (stencil
+// locality gives cache hits).  Up to eight entries per row
 // are loaded before the FMAs, so their gathers are in flight together, and
 // the chunks follow the slice width exactly (no predicated-off FP64 work).
 //
@@ -97,8 +97,8 @@ spmv_kernel(int n, int rows_per_cta, const int* __restrict__ rowptr,
 // is skipped per lane.
 template <int U, typename T>
 __device__ __forceinline__ void sell_chunk(const int* __restrict__ scol,
-                                           const T* __restrict__ sval,
-                                           const T* __restrict__ x, int k, T& sum) {
+                                           const T* __restrict__ sval, const T* x, int k,
+                                           T& sum) {
   int c[U];
   T v[U], xv[U];
 #pragma unroll
@@ -107,7 +107,7 @@ __device__ __forceinline__ void sell_chunk(const int* __restrict__ scol,
     v[u] = ld_stream(sval + k + 32 * u);
   }
 #pragma unroll
-  for (int u = 0; u < U; ++u) xv[u] = c[u] >= 0 ? __ldg(x + c[u]) : T(0);
+  for (int u = 0; u < U; ++u) xv[u] = c[u] >= 0 ? x[c[u]] : T(0);
 #pragma unroll
   for (int u = 0; u < U; ++u)
     if (c[u] >= 0) sum = fma(v[u], xv[u], sum);
@@ -120,8 +120,7 @@ __device__ __forceinline__ void sell_chunk(const int* __restrict__ scol,
 template <typename T>
 __device__ __forceinline__ T sell_row(const int* __restrict__ sptr,
                                       const int* __restrict__ scol,
-                                      const T* __restrict__ sval,
-                                      const T* __restrict__ x, int64_t row) {
+                                      const T* __restrict__ sval, const T* x, int64_t row) {
   const int64_t q = row >> 5;
   const int a = sptr[q], e = sptr[q + 1];
   const int w = (e - a) >> 5;
@@ -146,8 +145,8 @@ __device__ __forceinline__ T sell_row(const int* __restrict__ sptr,
 // (0xFFFF: padding).
 template <int U, typename T>
 __device__ __forceinline__ void sell_chunk16(int base, const uint16_t* __restrict__ soff,
-                                             const T* __restrict__ sval,
-                                             const T* __restrict__ x, int k, T& sum) {
+                                             const T* __restrict__ sval, const T* x, int k,
+                                             T& sum) {
   unsigned o[U];
   T v[U], xv[U];
 #pragma unroll
@@ -156,7 +155,7 @@ __device__ __forceinline__ void sell_chunk16(int base, const uint16_t* __restric
     v[u] = ld_stream(sval + k + 32 * u);
   }
 #pragma unroll
-  for (int u = 0; u < U; ++u) xv[u] = o[u] != 0xFFFFu ? __ldg(x + base + static_cast<int>(o[u])) : T(0);
+  for (int u = 0; u < U; ++u) xv[u] = o[u] != 0xFFFFu ? x[base + static_cast<int>(o[u])] : T(0);
 #pragma unroll
   for (int u = 0; u < U; ++u)
     if (o[u] != 0xFFFFu) sum = fma(v[u], xv[u], sum);
@@ -165,8 +164,7 @@ __device__ __forceinline__ void sell_chunk16(int base, const uint16_t* __restric
 template <typename T>
 __device__ __forceinline__ T sell_row16(const int* __restrict__ sptr, const int* __restrict__ sbase,
                                         const uint16_t* __restrict__ soff,
-                                        const T* __restrict__ sval, const T* __restrict__ x,
-                                        int64_t row) {
+                                        const T* __restrict__ sval, const T* x, int64_t row) {
   const int64_t q = row >> 5;
   const int a = sptr[q], e = sptr[q + 1];
   const int w = (e - a) >> 5;
@@ -195,9 +193,8 @@ __global__ void __launch_bounds__(kThreads)
 sell_kernel(int n, int64_t rows32, const int* __restrict__ sptr,
             const int* __restrict__ scol, const int* __restrict__ sbase,
             const uint16_t* __restrict__ soff, const int* __restrict__ sperm,
-            const T* __restrict__ sval, const T* __restrict__ x, const T* __restrict__ z,
-            T* __restrict__ y, T theta, T c, T inv_gamma) {
-  wait_previous();
+            const T* sval, const T* x, const T* z, T* __restrict__ y, T theta, T c, T inv_gamma) {
+  sval += wait_previous();
   release_next();
   for (int64_t pos = blockIdx.x * static_cast<int64_t>(kThreads) + threadIdx.x; pos < rows32;
        pos += static_cast<int64_t>(gridDim.x) * kThreads) {
