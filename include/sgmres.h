@@ -248,7 +248,15 @@ sg_status sg_mpk(sg_handle* h, const double* q, double* V, int64_t ldv,
  * the unit vector q (device, n doubles), in the handle's workspace, one
  * cooperative kernel per step (the launches of a k are captured once in a
  * CUDA graph and replayed).  precision: SG_PREC_FP64, or SG_PREC_FP32_IR
- * for the FP32 basis (q rounded to FP32).  H (host, ldh >= k+1, k columns,
+ * for the FP32 basis (q rounded to FP32).  FP64: where the largest
+ * magnitudes of A's rows lie within a factor 16 of one another and a share
+ * of w fits in each SM's shared memory (about 4.3M rows), the projections
+ * run in fixed point: an entry of a vector is held to 2^-58 of the largest
+ * one in its block of (at most 28K) rows, the coefficients are summed on a
+ * grid of 2^-70 ||A v_j||, in any order the same.  Relative to the vectors'
+ * norms that rounds less than FP64 does; an entry far below its block's
+ * largest has fewer bits than FP64 would keep.  Every other matrix takes the
+ * FP64 form, which keeps each entry's own 53 bits.  H (host, ldh >= k+1, k columns,
  * column-major) receives the (k+1) x k Hessenberg matrix, *steps the steps
  * completed (fewer than k after an invariant subspace: h_{j+1,j} <= 1e-12
  * of ||A v_j||).  Synchronises `stream`.  Errors: SG_EINVAL (k < 1, null

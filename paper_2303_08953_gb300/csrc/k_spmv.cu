@@ -28,8 +28,10 @@
 // contiguous block of rows and first stages that block's values and
 // column indices in shared memory with coalesced streaming loads, then
 // each thread walks its own row from shared memory.
+#include <cstring>
 #include <map>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "k_reduce.cuh"
@@ -460,12 +462,109 @@ arnoldi_step_kernel(int n, int rows_per_cta, const int* __restrict__ rowptr,
     w[i] = static_cast<T>(static_cast<double>(w[i]) * inv);
 }
 
-// The same FP64 step with w resident on chip, in fixed point.  w = A v_j is
-// first formed in V's column j+1 by the SELL SpMV kernel (full occupancy,
-// and the whole L1 for the gathers of v_j); then CTA b of this cooperative
-// kernel loads its rows [b R, (b+1) R) of w into shared memory and keeps
-// them there through the projections to the final normalisation, streaming
-// the vectors past them.
+// The FP64 step with w resident on chip.  w = A v_j is first formed in V's
+// column j+1 by the SpMV kernel (full occupancy, and the whole L1 for the
+// gathers of v_j); then CTA b of this cooperative kernel loads its rows
+// [b R, (b+1) R) of w into shared memory and keeps them there through the
+// MGS phases to the final normalisation.  A thread always touches the same
+// rows, so w needs no barrier of its own; each phase streams only v_l (just
+// read as the previous phase's v_{l+1}, an L2 hit) and v_{l+1}, instead of
+// reading and writing w through HBM as well.  Phase order, fused next-vector
+// dot and per-CTA partials are those of arnoldi_step_kernel; only the rows a
+// CTA owns differ.  It runs for the matrices that the fixed-point step below
+// is not for (rows_even): whole pre-pass with its products, 60 steps at 149K
+// rows 10.9 ms (fixed point 4.66), at 2.10M rows 25.2 ms (14.1), 40 steps at
+// 400K rows in CSR 9.4 ms (6.5; arnoldi_step_kernel 10.6).  The FP64 pipe
+// bounds it.
+__global__ void __launch_bounds__(kCoopThreads, 1)
+arnoldi_mgs_resident64_kernel(int n, int rows_cta, double* __restrict__ V, int64_t ld, int j,
+                              double* __restrict__ H, int ldh, double* __restrict__ wn,
+                              double* __restrict__ red, unsigned* ctr, unsigned base, int* err) {
+  extern __shared__ __align__(16) unsigned char coop_smem[];
+  double* ws = reinterpret_cast<double*>(coop_smem);
+  const int G = gridDim.x;
+  const int t = threadIdx.x;
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * rows_cta;
+  const int64_t r1 = (r0 + rows_cta < n) ? r0 + rows_cta : n;
+  const int nr = r1 > r0 ? static_cast<int>(r1 - r0) : 0;
+  const double* v0 = V + r0;
+  double* w = V + static_cast<int64_t>(j + 1) * ld + r0;
+  double* pWW = red;
+  double* pA = red + G;
+  double* pB = red + 2 * G;
+  // this CTA's rows of w = A v_j, partials of w.w and v_0.w
+  double accw = 0.0, accv = 0.0;
+  for (int i = t; i < nr; i += kCoopThreads) {
+    const double wi = w[i];
+    ws[i] = wi;
+    accw = fma(wi, wi, accw);
+    accv = fma(v0[i], wi, accv);
+  }
+  {
+    const double sw = block_sum_few_d<kCoopThreads>(accw);
+    const double sv = block_sum_few_d<kCoopThreads>(accv);
+    if (t == 0) { pWW[blockIdx.x] = sw; pA[blockIdx.x] = sv; }
+  }
+  unsigned target = base + static_cast<unsigned>(G);
+  grid_barrier_count(ctr, target, err);
+  if (blockIdx.x == 0) {
+    const double ww = sum_partials_few_d<kCoopThreads>(pWW, G);
+    if (t == 0) wn[j] = sqrt(ww);
+  }
+  // MGS phases l = 0..j: h_l from the previous phase's partials, w -= h_l
+  // v_l, partials of v_{l+1}.w (of w.w in the last phase)
+  double* pin = pA;
+  double* pout = pB;
+  for (int l = 0; l <= j; ++l) {
+    const double h = sum_partials_few_d<kCoopThreads>(pin, G);
+    if (blockIdx.x == 0 && t == 0) H[l + static_cast<int64_t>(j) * ldh] = h;
+    const double* vl = V + static_cast<int64_t>(l) * ld + r0;
+    const double* vn = V + static_cast<int64_t>(l + 1) * ld + r0;
+    double acc = 0.0;
+    int i = t;
+    if (l < j) {
+      for (; i + 3 * kCoopThreads < nr; i += 4 * kCoopThreads) {
+        double wv[4], vv[4], nv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          wv[u] = ws[i + u * kCoopThreads];
+          vv[u] = vl[i + u * kCoopThreads];
+          nv[u] = vn[i + u * kCoopThreads];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const double wi = fma(-h, vv[u], wv[u]);
+          ws[i + u * kCoopThreads] = wi;
+          acc = fma(nv[u], wi, acc);
+        }
+      }
+      for (; i < nr; i += kCoopThreads) {
+        const double wi = fma(-h, vl[i], ws[i]);
+        ws[i] = wi;
+        acc = fma(vn[i], wi, acc);
+      }
+    } else {
+      for (; i < nr; i += kCoopThreads) {
+        const double wi = fma(-h, vl[i], ws[i]);
+        ws[i] = wi;
+        acc = fma(wi, wi, acc);
+      }
+    }
+    const double tot = block_sum_few_d<kCoopThreads>(acc);
+    if (t == 0) pout[blockIdx.x] = tot;
+    target += static_cast<unsigned>(G);
+    grid_barrier_count(ctr, target, err);
+    double* tmp = pin; pin = pout; pout = tmp;
+  }
+  // normalise into V's column j+1
+  const double nrm = sqrt(sum_partials_few_d<kCoopThreads>(pin, G));
+  if (blockIdx.x == 0 && t == 0) H[(j + 1) + static_cast<int64_t>(j) * ldh] = nrm;
+  const double inv = 1.0 / nrm;
+  for (int i = t; i < nr; i += kCoopThreads) w[i] = ws[i] * inv;
+}
+
+// The same step in fixed point: w resident as above, the vectors streamed
+// past it, for matrices whose rows are of like size (rows_even).
 //
 // In FP64 the FP64 pipe bounds a projection (two FMAs a row at 2 a clock and
 // SM: 13 of 20 us at 4.19M rows, where the vector takes 5 us from HBM), then
@@ -480,8 +579,12 @@ arnoldi_step_kernel(int n, int rows_per_cta, const int* __restrict__ rowptr,
 //       w -= h v:  h 2^ev in units of w, rounded to an integer, times v 2^-60,
 //             rounded to w's unit.
 //     The unit of v is 2^-58 of the CTA's largest entry or less, that of w
-//     2^-60 or less at the start: the projections round less than FP64 ones
-//     do.  Since |w| can grow while it is projected, its bound grows by
+//     2^-60 or less at the start: relative to the vectors' norms the
+//     projections round less than FP64 ones do, but an entry far below its
+//     CTA's largest keeps fewer bits than FP64's 53 (below 2^-60 of it,
+//     none).  That matters where the next product with A multiplies small
+//     entries by large ones, and rows_even leaves those matrices to FP64.
+//     Since |w| can grow while it is projected, its bound grows by
 //     |h| 2^ev per projection and w is shifted down when the bound reaches
 //     2^61 units.
 //   * the CTAs' partial sums are added with integer atomics on a common grid
@@ -1819,30 +1922,32 @@ bool launch_arnoldi_icwy(const DevCsr& A, const float* val, float* V, int64_t ld
   return true;
 }
 
-// Rows per CTA of the resident FP64 step for n rows, or 0 when a CTA's
-// slice of w would not fit in shared memory next to the kernel's static
+// Rows per CTA of a resident FP64 step's kernel fn for n rows, or 0 when a
+// CTA's slice of w would not fit in shared memory next to the kernel's static
 // reduction buffers (then the streaming step runs).  One CTA per SM, at
-// least 1024 rows per CTA (fewer CTAs, cheaper exchanges, on small systems).
-int resident_rows_per_cta(int64_t n, int* grid) {
+// least min_rows rows per CTA (fewer CTAs, cheaper exchanges, on small
+// systems).
+int resident_rows_per_cta(int64_t n, const void* fn, int min_rows, int* grid) {
   static std::mutex mu;
-  static std::map<int, int> limit;   // device -> dynamic bytes available
+  static std::map<std::pair<int, const void*>, int> limit;   // dynamic bytes available
   const int dev = current_device();
   int avail;
   {
     std::lock_guard<std::mutex> lock(mu);
-    auto it = limit.find(dev);
+    auto it = limit.find({dev, fn});
     if (it == limit.end()) {
       int optin = 0;
       SG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
       cudaFuncAttributes fa{};
-      SG_CUDA(cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(arnoldi_mgs_resident_kernel)));
-      it = limit.emplace(dev, optin - static_cast<int>(fa.sharedSizeBytes) - 1024).first;
+      SG_CUDA(cudaFuncGetAttributes(&fa, fn));
+      it = limit.emplace(std::make_pair(dev, fn),
+                         optin - static_cast<int>(fa.sharedSizeBytes) - 1024).first;
     }
     avail = it->second;
   }
   const int64_t sms = device_sm_count();
   int64_t R = (n + sms - 1) / sms;
-  if (R < 1024) R = 1024;
+  if (R < min_rows) R = min_rows;
   R = (R + 31) / 32 * 32;
   if (R * static_cast<int64_t>(sizeof(double)) > avail) return 0;
   *grid = static_cast<int>((n + R - 1) / R);
@@ -1861,9 +1966,9 @@ void launch_arnoldi_step(const DevCsr& A, const T* val, T* V, int64_t ld, int j,
                          unsigned* bar, int* err, cudaStream_t st) {
   if constexpr (sizeof(T) == 8) {
     int G = 0;
-    const int R = resident_rows_per_cta(A.n, &G);
-    if (R > 0 && G <= device_sm_count() && G < 256 && xv && fixed_red_doubles(G, k) <= red_cap) {
-      const void* fn = reinterpret_cast<const void*>(arnoldi_mgs_resident_kernel);
+    const void* fn = reinterpret_cast<const void*>(arnoldi_mgs_resident_kernel);
+    int R = A.rows_even == 1 && xv ? resident_rows_per_cta(A.n, fn, 1024, &G) : 0;
+    if (R > 0 && G <= device_sm_count() && G < 256 && fixed_red_doubles(G, k) <= red_cap) {
       const int smem = R * static_cast<int>(sizeof(double));
       ensure_dynamic_smem(fn, smem);
       int per_sm = 0;
@@ -1889,6 +1994,32 @@ void launch_arnoldi_step(const DevCsr& A, const T* val, T* V, int64_t ld, int j,
         int rc = R;
         void* args[] = {&n, &rc, &V, &ld, &j, &xv, &H, const_cast<int*>(&ldh), &wn, &fs, &err};
         SG_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kFxThreads), args, smem, st));
+        count_launch();
+        return;
+      }
+    }
+    fn = reinterpret_cast<const void*>(arnoldi_mgs_resident64_kernel);
+    R = A.rows_even != 1 ? resident_rows_per_cta(A.n, fn, 2048, &G) : 0;
+    if (R > 0 && G <= device_sm_count() && 3 * G <= red_cap) {
+      const int smem = R * static_cast<int>(sizeof(double));
+      ensure_dynamic_smem(fn, smem);
+      int per_sm = 0;
+      SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kCoopThreads, smem));
+      if (per_sm >= 1) {
+        // w = A v_j into V's column j+1, then the MGS phases on chip
+        dispatch<0, false, T>(A, A.val, A.sval, V + static_cast<int64_t>(j) * ld, nullptr,
+                              V + static_cast<int64_t>(j + 1) * ld, T(0), T(0), T(1), st);
+        // barriers per step j: one after the w partials, one per MGS phase
+        // (j + 1); the counter (word 16 of the barrier block, zeroed at the
+        // start of the pre-pass) has seen G (j' + 2) arrivals per earlier step
+        int n = A.n;
+        int rc = R;
+        unsigned* ctr = bar + 16;
+        unsigned base = static_cast<unsigned>(G) * static_cast<unsigned>(j) *
+                        static_cast<unsigned>(j + 3) / 2u;
+        void* args[] = {&n, &rc, &V, &ld, &j, &H, const_cast<int*>(&ldh), &wn, &red, &ctr,
+                        &base, &err};
+        SG_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kCoopThreads), args, smem, st));
         count_launch();
         return;
       }
@@ -1946,6 +2077,58 @@ __global__ void sampled_outer_kernel(int n, const int* __restrict__ rowptr,
     const double li = -lam[row];
     const int s = rowptr[row], e = rowptr[row + 1];
     for (int k = s + l; k < e; k += VEC) dval[k] = li * __ldg(x + colind[k]);
+  }
+}
+
+// Largest magnitudes of the rows (eight lanes per row), as bit patterns: of
+// those, out[0] the largest and out[1] the complement of the smallest (both 0
+// before).  An infinity or NaN has the largest pattern.
+__global__ void __launch_bounds__(kThreads)
+row_extent_kernel(int n, const int* __restrict__ rowptr, const double* __restrict__ val,
+                  unsigned long long* out) {
+  constexpr int VEC = 8;
+  __shared__ unsigned long long sh[2][kThreads / 32];
+  const int l = threadIdx.x % VEC;
+  unsigned long long hi = 0, lo = 0;
+  // (every lane of a warp takes the same number of turns)
+  for (int64_t r0 = static_cast<int64_t>(blockIdx.x) * kThreads / VEC; r0 < n;
+       r0 += static_cast<int64_t>(gridDim.x) * kThreads / VEC) {
+    const int64_t r = r0 + threadIdx.x / VEC;
+    unsigned long long m = 0;
+    if (r < n) {
+      const int e = rowptr[r + 1];
+      for (int k = rowptr[r] + l; k < e; k += VEC) {
+        const unsigned long long b =
+            static_cast<unsigned long long>(__double_as_longlong(val[k])) & 0x7FFFFFFFFFFFFFFFull;
+        m = b > m ? b : m;
+      }
+    }
+#pragma unroll
+    for (int off = VEC / 2; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, off);
+      m = o > m ? o : m;
+    }
+    if (r < n) {
+      hi = m > hi ? m : hi;
+      lo = ~m > lo ? ~m : lo;
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    unsigned long long o = __shfl_xor_sync(0xffffffffu, hi, off);
+    hi = o > hi ? o : hi;
+    o = __shfl_xor_sync(0xffffffffu, lo, off);
+    lo = o > lo ? o : lo;
+  }
+  if (threadIdx.x % 32 == 0) {
+    sh[0][threadIdx.x / 32] = hi;
+    sh[1][threadIdx.x / 32] = lo;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    unsigned long long m = 0;
+    for (int w = 0; w < kThreads / 32; ++w) m = sh[threadIdx.x][w] > m ? sh[threadIdx.x][w] : m;
+    atomicMax(out + threadIdx.x, m);
   }
 }
 
@@ -2518,6 +2701,39 @@ void scale_columns(const DevCsr& A, const double* d, DevCsr& E, cudaStream_t st)
     scale_cols_kernel<<<g, kThreads, 0, st>>>(A.sell_nnz, A.scol, A.sval, d, E.sval);
     SG_LAUNCH_CHECK();
   }
+}
+
+void row_extent(const DevCsr& A, unsigned long long* out, cudaStream_t st) {
+  SG_CUDA(cudaMemsetAsync(out, 0, 2 * sizeof(unsigned long long), st));
+  int64_t blocks = (static_cast<int64_t>(A.n) * 8 + kThreads - 1) / kThreads;
+  const int64_t cap = static_cast<int64_t>(device_sm_count()) * 8;
+  if (blocks > cap) blocks = cap;
+  row_extent_kernel<<<static_cast<unsigned>(blocks), kThreads, 0, st>>>(A.n, A.rowptr, A.val, out);
+  SG_LAUNCH_CHECK();
+}
+
+// The fixed-point pre-pass step holds an entry of a vector to about 2^-58 of
+// its CTA's largest one, FP64 to 2^-53 of itself.  The loss in v_j comes back
+// multiplied by A's entries, so it shows in H where an entry of A is large
+// against the product's size.  If the largest magnitudes of all rows lie
+// within a factor f, that cannot be: following each row's largest entry from
+// row to row ends in a cycle, so |A| restricted to any set of rows that is
+// closed under it has a spectral radius of at least max|a| / f.  D B D^-1
+// with random powers of two in D, the 32^2 and 150 x 101 stencils, 20 and 8
+// steps, the largest error of H relative to its column's largest entry,
+// fixed point against FP64, by f:
+//   1: 5e-15, 5e-15     2^2: 5e-15, 1e-14    2^4: 5e-15, 5e-15
+//   2^6: 1e-14, 7e-15   2^8: 5e-14, 1e-14    2^18: 4e-11, 9e-15
+// so the line lies at 16 (a matrix of zero rows, infinities or NaN is beyond
+// it too).  Rows or columns scaled alone lose nothing in fixed point up to
+// 2^50; they go to FP64 by this rule all the same.
+bool rows_are_even(const unsigned long long* out) {
+  const unsigned long long hi = out[0], lo = ~out[1];
+  if (lo == 0 || hi >= 0x7FF0000000000000ull) return false;
+  double a, b;
+  std::memcpy(&a, &hi, sizeof(a));
+  std::memcpy(&b, &lo, sizeof(b));
+  return a <= 16.0 * b;
 }
 
 void diag_apply(int64_t n, const double* d, const double* x, double* y, bool div,

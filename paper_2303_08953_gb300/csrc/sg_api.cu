@@ -210,6 +210,7 @@ void ensure_transpose(sg_handle* h, cudaStream_t st) {
   } else {
     sg::transpose_values(h->A, T, st);
     sg::sell_refill_values(T, st);
+    T.rows_even = -1;
   }
   if (T.val32 || h->A.val32) make_val32(T, st);
   h->at_stale = false;
@@ -240,6 +241,7 @@ void ensure_equil(sg_handle* h, cudaStream_t st) {
     E = h->A;  // pattern arrays are shared with A
     E.val = E.sval = nullptr;
     E.val32 = E.sval32 = nullptr;
+    E.rows_even = -1;
     SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&E.val), sizeof(double) * std::max<int64_t>(h->A.nnz, 1)));
     if (h->A.sptr)
       SG_CUDA(cudaMalloc(reinterpret_cast<void**>(&E.sval), sizeof(double) * h->A.sell_nnz));
@@ -482,6 +484,7 @@ sg_status sg_update_values(sg_handle* h, const double* val, int32_t on_device) {
     if (h->A.nnz) copy_in(h->A.val, val, h->A.nnz, on_device != 0, st);
     sg::sell_refill_values(h->A, st);
     if (h->A.val32) make_val32(h->A, st);
+    h->A.rows_even = -1;
     h->at_stale = true;  // the transpose takes them over on its next use
     SG_CUDA(cudaStreamSynchronize(st));
   });

@@ -66,6 +66,9 @@ struct DevCsr {
   uint16_t* soff = nullptr;
   // A transpose's entry p holds the value of entry src[p] of the original.
   int32_t* src = nullptr;
+  // Whether the rows' largest magnitudes lie close together (rows_are_even):
+  // 1 or 0, -1 while not known for the present values.
+  mutable int rows_even = -1;
 };
 
 // Build A's SELL-32 copy from its CSR arrays, with the rows in order or, when
@@ -104,8 +107,9 @@ void spmv_newton32(const DevCsr& A, const float* x, const float* z, float* y,
 // one V, xv and red); red: >= prepass_red_doubles(k) doubles; bar: 64 zeroed
 // unsigned words (barrier state); err: set to 1 if a barrier wait ran out.
 // FP64: xv (one column) receives each new vector in FP64 while V holds them
-// in fixed point, on systems whose w stays in shared memory; elsewhere V
-// holds FP64 columns and xv is not used.
+// in fixed point, on systems whose w stays in shared memory and whose rows
+// are even (A.rows_even == 1); elsewhere V holds FP64 columns and xv is not
+// used.
 void arnoldi_step(const DevCsr& A, double* V, int64_t ld, int j, int k, double* xv, double* H,
                   int ldh, double* wn, double* red, int red_cap, unsigned* bar,
                   int* err, cudaStream_t st);
@@ -117,6 +121,11 @@ void arnoldi_step32(const DevCsr& A, float* V, int64_t ld, int j, double* H,
                     int ldh, double* wn, double* red, int red_cap, unsigned* bar,
                     int* err, cudaStream_t st);
 int64_t prepass_red_doubles(int k);
+// The largest magnitudes of A's rows: out[0] (device) receives the largest of
+// them, out[1] the complement of the smallest, as bit patterns; rows_are_even
+// on their host copy says whether the FP64 pre-pass may run in fixed point.
+void row_extent(const DevCsr& A, unsigned long long* out, cudaStream_t st);
+bool rows_are_even(const unsigned long long* out);
 // r = b - A x
 void residual(const DevCsr& A, const double* b, const double* x, double* r,
               cudaStream_t st);

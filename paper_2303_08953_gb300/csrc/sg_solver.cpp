@@ -241,6 +241,20 @@ unsigned* prepass_barrier(sg_handle* h) {
 }
 int* prepass_error(sg_handle* h) { return reinterpret_cast<int*>(prepass_barrier(h) + 48); }
 
+// Extent of the rows of M, by way of the scalar slots: enqueued, and taken
+// over once the stream has been synchronised.
+unsigned long long* extent_slot(sg_handle* h, double* base) {
+  return reinterpret_cast<unsigned long long*>(base + slots_for(h->ws_m, h->ws_k).scal + 8);
+}
+void fetch_row_extent(sg_handle* h, const DevCsr& M, cudaStream_t st) {
+  row_extent(M, extent_slot(h, h->small), st);
+  SG_CUDA(cudaMemcpyAsync(extent_slot(h, h->hbuf), extent_slot(h, h->small),
+                          2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+}
+void take_row_extent(sg_handle* h, const DevCsr& M) {
+  M.rows_even = rows_are_even(extent_slot(h, h->hbuf)) ? 1 : 0;
+}
+
 template <typename T>
 void enqueue_prepass(sg_handle* h, const DevCsr& M, const T* q, int k,
                      cudaStream_t st) {
@@ -274,13 +288,20 @@ int arnoldi_prepass(sg_handle* h, const DevCsr& M, const T* q, int k,
   const void* key[6] = {M.sptr ? static_cast<const void*>(M.sptr) : M.rowptr, vals, q,
                         B::V(h), h->small, h->red};
   prepass_barrier(h);  // allocate the barrier block before any capture
+  if (sizeof(T) == 8 && M.rows_even < 0) {
+    fetch_row_extent(h, M, st);
+    SG_CUDA(cudaStreamSynchronize(st));
+    take_row_extent(h, M);
+  }
+  const int form = sizeof(T) == 8 ? M.rows_even : 0;
   sg_handle::PrepassGraph* g = nullptr;
   for (auto& c : h->graphs)
-    if (c.k == k && c.n == M.n && std::equal(key, key + 6, c.key)) g = &c;
+    if (c.k == k && c.n == M.n && c.form == form && std::equal(key, key + 6, c.key)) g = &c;
   if (!g) {
     sg_handle::PrepassGraph ng;
     std::copy(key, key + 6, ng.key);
     ng.k = k;
+    ng.form = form;
     ng.n = M.n;
     cudaGraph_t graph = nullptr;
     const long long before = launches_so_far();
@@ -457,7 +478,11 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
   residual(M, h->bvec, h->xvec, h->rvec, st);
   device_norm(h->rvec, sc);
   fetch(sc, 1, hb);
+  // (what the FP64 pre-pass's form depends on, under the same synchronisation)
+  const bool extent = sizeof(T) == 8 && o.n_ritz == 0 && M.rows_even < 0;
+  if (extent) fetch_row_extent(h, M, st);
   SG_CUDA(cudaStreamSynchronize(st));
+  if (extent) take_row_extent(h, M);
   const double beta0 = hb[0];
   log = SolveLog();
   if (!std::isfinite(beta0)) throw Error(SG_ENUMERIC, "non-finite initial residual");

@@ -48,6 +48,7 @@ struct sg_handle {
   struct PrepassGraph {
     const void* key[6];
     int k = 0;
+    int form = 0;            // FP64: M.rows_even, which picks the step's form
     int64_t n = 0;
     long long kernels = 0;
     cudaGraphExec_t exec = nullptr;
