@@ -374,9 +374,16 @@ int64_t sg_kernel_launches(void);
  * the FP64 pipe; SG_TC_NEVER (1): always the FP64-pipe kernels (also what
  * the environment variable SGMRES_NO_TC=1 selects at the first call);
  * SG_TC_ALWAYS (2): the tensor-core form wherever its layout requirements
- * hold.  Both forms give the same products to FP64 rounding, so this only
- * chooses speed.  Process-wide; returns the previous policy, or -1 for an
- * unknown value (nothing changed). */
+ * hold.  The tensor-core form adds 62-bit integers exactly and rounds once;
+ * it holds a value to 2^-62 of the largest finite one in its column (of Q, X,
+ * and of W with row k scaled by column k of Q), so for columns of like
+ * magnitudes it is the more accurate one, while entries more than 2^9 below
+ * their column's largest have fewer bits than FP64's 53, and a row of Q below
+ * 2^-62 of every column's largest adds nothing to an update; subnormal
+ * values count as zero.  In both forms an Inf or a NaN makes the outputs that
+ * it enters non-finite (NaN on the tensor cores) and no others.
+ * Process-wide; returns the previous policy, or -1 for an unknown value
+ * (nothing changed). */
 #define SG_TC_AUTO 0
 #define SG_TC_NEVER 1
 #define SG_TC_ALWAYS 2

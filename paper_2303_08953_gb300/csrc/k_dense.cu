@@ -213,9 +213,12 @@ dot_small_kernel(int64_t K, int M, int N, const double* A, int64_t lda,
 // W(m, n) = sum_z part[z](m, n); sym reads the upper element for both
 // (m, n) and (n, m).  One warp per output: lane l adds splits l, l+32, ...
 // in order, then a fixed xor-shuffle tree combines the lanes, so the
-// result is deterministic and the S loads are issued 32 at a time.
+// result is deterministic and the S loads are issued 32 at a time.  fa, fb:
+// null, or the columns' exponent pairs of a digit-slice product, whose
+// non-finite columns (.y > 0) give NaN here.
 __global__ void reduce_parts_kernel(int M, int N, int S, const double* part,
-                                    double* __restrict__ W, int ldw, int sym) {
+                                    double* __restrict__ W, int ldw, int sym, const int2* fa,
+                                    const int2* fb) {
   wait_previous();
   release_next();
   const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -224,20 +227,22 @@ __global__ void reduce_parts_kernel(int M, int N, int S, const double* part,
   const int m = static_cast<int>(gw % M), n = static_cast<int>(gw / M);
   int sm = m, sn = n;
   if (sym && m > n) { sm = n; sn = m; }
+  const bool bad = fa && (fa[m].y > 0 || fb[n].y > 0);
   double acc = 0.0;
   const int64_t MN = static_cast<int64_t>(M) * N;
   const double* p = part + sm + static_cast<int64_t>(sn) * M;
   for (int z = lane; z < S; z += 32) acc += p[z * MN];
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (lane == 0) W[m + static_cast<int64_t>(n) * ldw] = acc;
+  if (lane == 0)
+    W[m + static_cast<int64_t>(n) * ldw] = bad ? __longlong_as_double(0x7FF8000000000000ll) : acc;
 }
 
 void launch_reduce(int M, int N, int S, const double* part, double* W, int ldw,
-                   bool sym, cudaStream_t st) {
+                   bool sym, cudaStream_t st, const int2* fa = nullptr, const int2* fb = nullptr) {
   const int64_t threads = static_cast<int64_t>(M) * N * 32;
   launch_early(true, reduce_parts_kernel, dim3(static_cast<unsigned>((threads + 255) / 256)), 256, 0,
-               st, M, N, S, part, W, ldw, sym ? 1 : 0);
+               st, M, N, S, part, W, ldw, sym ? 1 : 0, fa, fb);
   SG_LAUNCH_CHECK();
 }
 
@@ -505,12 +510,13 @@ void block_dot_impl(int64_t n, const T* Q, int64_t ldq, int i, const T* X,
     // exponents sit after the split partials.  A Gram comes out exactly
     // symmetric (both triangles are the same exact sums).
     const int64_t need = oz_dot_part_size(n, i, s);
-    SG_REQUIRE(need + (oz_exp_ints(i, s) + 1) / 2 <= part_cap, SG_EINVAL,
+    SG_REQUIRE(need + oz_exp_doubles(i, s) <= part_cap, SG_EINVAL,
                "block_dot: workspace too small");
     int S = 0;
+    const int2 *fq = nullptr, *fx = nullptr;
     oz_dot(n, reinterpret_cast<const double*>(Q), ldq, i, reinterpret_cast<const double*>(X),
-           ldx, s, reinterpret_cast<int*>(part + need), part, need, &S, st, eq, ex);
-    launch_reduce(i, s, S, part, W, ldw, false, st);
+           ldx, s, reinterpret_cast<int2*>(part + need), part, need, &S, st, eq, ex, &fq, &fx);
+    launch_reduce(i, s, S, part, W, ldw, false, st, fq, fx);
     return;
   }
   if (sizeof(T) == 8 && small_dot(i, s, sym)) {
@@ -954,7 +960,7 @@ int64_t block_dot_part_size(int64_t n, int i, int s) {
     if (g > need) need = g;
   }
   const int64_t tc = tc_dot_part_size(n, i, s);
-  const int64_t oz = oz_dot_part_size(n, i, s) + (oz_exp_ints(i, s) + 1) / 2;
+  const int64_t oz = oz_dot_part_size(n, i, s) + oz_exp_doubles(i, s);
   need = need > tc ? need : tc;
   return need > oz ? need : oz;
 }
@@ -974,7 +980,7 @@ void block_dot32(int64_t n, const float* Q, int64_t ldq, int i,
                         st);
 }
 
-int64_t block_update_scratch(int i) { return (static_cast<int64_t>(i) + 1) / 2 + 1; }
+int64_t block_update_scratch(int i) { return oz_exp_doubles(i, 0) + 1; }
 
 void block_update(int64_t n, const double* Q, int64_t ldq, int i,
                   const double* W, int ldw, double* X, int64_t ldx, int s,
@@ -985,7 +991,7 @@ void block_update(int64_t n, const double* Q, int64_t ldq, int i,
       (tc_forced() || oz_update_pays(n, i, s, upper))) {
     // FP64 products on the tensor cores, exact digit slices
     oz_update(n, Q, ldq, i, W, ldw, X, ldx, s, alpha, beta, upper,
-              reinterpret_cast<int*>(scratch), st, eq, ex);
+              reinterpret_cast<int2*>(scratch), st, eq, ex);
     return;
   }
   if (ex) ex->valid = 0;

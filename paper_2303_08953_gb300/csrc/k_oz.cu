@@ -123,8 +123,8 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t d) {
 // truncated, plus 0x80 in every byte: the mantissa with its top bit at bit
 // 61 is shifted right by e + 1022 - E (E: the exponent field).  Zeros and
 // subnormals (E = 0) give m = 0, and so does every shift outside 0 .. 63
-// (infinities and NaN, whose columns' exponents are those of finite values;
-// columns without an exponent).
+// (infinities and NaN, whose columns' exponents are those of finite values
+// and whose outputs become NaN outside the sums; columns without an exponent).
 __device__ __forceinline__ uint2 biased62(double x, int e) {
   const uint32_t xh = static_cast<uint32_t>(__double2hiint(x));
   const uint32_t xl = static_cast<uint32_t>(__double2loint(x));
@@ -175,6 +175,11 @@ __device__ __forceinline__ uint32_t near_word(int e) {
 
 __device__ __forceinline__ uint32_t near_test(double x, uint32_t w) {
   return w - 2u * static_cast<uint32_t>(__double2hiint(x));
+}
+
+// an Inf or a NaN
+__device__ __forceinline__ bool non_finite(double x) {
+  return (static_cast<uint32_t>(__double2hiint(x)) & 0x7FF00000u) == 0x7FF00000u;
 }
 
 // Balanced base-256 digits of two numbers as FP16 pairs: w[t] holds digit
@@ -371,7 +376,7 @@ constexpr int kUSplit = kUWarps * 32;
 __global__ void __launch_bounds__(kDThreads, 1)
 oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
               const __grid_constant__ CUtensorMap mapX, int64_t n, int M, int N,
-              const int* __restrict__ eq, const int* __restrict__ ex, int64_t rows_per_split,
+              const int2* __restrict__ eq, const int2* __restrict__ ex, int64_t rows_per_split,
               double* __restrict__ part, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char dsmem[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
@@ -513,8 +518,8 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
     // B (X, into shared-memory slices): warp w takes rows 2w, 2w + 1 of all
     // 32 columns (box w / 8, chunk w % 8), lane = column.
     const int m = (warp & 3) * 32 + lane;    // Q column m0 + m
-    const int eM = (m0 + m < M) ? eq[m0 + m] : -4000;
-    const int eN = (n0 + lane < N) ? ex[n0 + lane] : -4000;
+    const int eM = (m0 + m < M) ? eq[m0 + m].x : -4000;
+    const int eN = (n0 + lane < N) ? ex[n0 + lane].x : -4000;
     const uint32_t tlane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     const uint32_t wM = near_word(eM), wN = near_word(eN);
     const uint32_t one = blockDim.z;   // 1
@@ -606,7 +611,7 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
     const int gm = m0 + (warp & 3) * 32 + lane;
     if (gm < M) {
       double* P = part + static_cast<int64_t>(blockIdx.z) * M * N;
-      const int eM = eq[gm];
+      const int eM = eq[gm].x;
 #pragma unroll
       for (int cc = 0; cc < kCols; ++cc) {
         const int gc = n0 + cg * kCols + cc;
@@ -614,8 +619,9 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
           // V' = (ahi + carry) 2^32 + the low 32 bits of alo, rounded once
           const int64_t hi = static_cast<int64_t>(ahi[cc]) + (static_cast<int64_t>(alo[cc]) >> 32);
           const uint32_t lo = static_cast<uint32_t>(alo[cc]);
+          const int eN = ex[gc].x;
           P[gm + static_cast<int64_t>(gc) * M] =
-              (eM < -2000 || ex[gc] < -2000) ? 0.0 : int96_to_double(hi, lo, eM + ex[gc] - 68);
+              (eM < -2000 || eN < -2000) ? 0.0 : int96_to_double(hi, lo, eM + eN - 68);
         }
       }
     }
@@ -676,7 +682,7 @@ constexpr uint32_t kUACol = 256;                        // A buffer b: 256 + 128
 // e_k, W' column exponents g_c
 struct OzUTables {
   alignas(16) uint32_t w[kUMaxK];
-  uint32_t top[kUN];               // largest finite |x|'s high word per output column
+  uint32_t top[kUN];               // largest |x|'s high word per output column
   int g[kUN];
 };
 
@@ -685,7 +691,9 @@ struct __align__(8) OzUShared {
   uint64_t accfull, accfree, xfull, xfree, done;
   uint32_t tmem_base;
   int fail;
+  int bad;                         // Q or W' holds an Inf or a NaN
 };
+constexpr int kUNonFinite = 1 << 20;   // "exponent" of a column of W' that holds one
 
 // dynamic shared memory: Q ring, X box, W' slices, tables, barriers (all of
 // it dynamic, so the 1 KB alignment slack fits under the 227 KB limit)
@@ -711,13 +719,34 @@ __host__ __device__ inline int oz_update_first(int ct, int ntc, int i, int upper
   return ct + static_cast<int>((P - ntc) * before / all);
 }
 
+// NaN for the rows of a CTA's tiles whose row of Q holds an Inf or a NaN, and
+// for the columns of which W' does (g: the tile's column exponents).
+__device__ __noinline__ void update_non_finite(int64_t n, int i, int s, const double* Q, int64_t ldq,
+                                               double* X, int64_t ldx, int n0, int g0, int G,
+                                               const int* g, int2* eout) {
+  if (threadIdx.x >= kUSplit) return;
+  const int c0 = n0 + kUN / 4 * (static_cast<int>(threadIdx.x) >> 7);
+  for (int64_t rt = g0; rt * kUM < n; rt += G) {
+    const int64_t r = rt * kUM + (threadIdx.x & 127);
+    if (r >= n) break;
+    bool row = false;
+    for (int k = 0; k < i; ++k) row = row || non_finite(Q[r + k * ldq]);
+    for (int c = c0; c < c0 + kUN / 4 && c < s; ++c)
+      if (row || g[c - n0] == kUNonFinite) {
+        X[r + c * ldx] = __longlong_as_double(0x7FF8000000000000ll);
+        if (eout) eout[c].y = 1;
+      }
+  }
+}
+
 // grid: CTAs of every column tile in turn; the g-th of a tile's G takes row
 // tiles g, g + G, ...
 __global__ void __launch_bounds__(kUThreads, 1)
 oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapX,
                  int64_t n, int i, int s, const double* __restrict__ W, int ldw,
                  double* __restrict__ X, int64_t ldx, double alpha, double beta, int upper,
-                 const int* __restrict__ eq, int* __restrict__ eout, int* __restrict__ err) {
+                 const int2* __restrict__ eq, int2* __restrict__ eout, const double* Q, int64_t ldq,
+                 int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char dsmem[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -769,6 +798,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     mbar_init(&sh.xfree, kUSplit);
     mbar_init(&sh.done, 1);
     sh.fail = 0;
+    sh.bad = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -782,7 +812,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   // W' = W 2^(e_k) (zero below the diagonal when `upper`) cut into digits
   // relative to its column exponents g_c: B slices of every 64 columns of Q
   if (warp < kUWarps) {
-    for (int k = tid; k < kUMaxK; k += kUSplit) tb.w[k] = near_word(k < i ? eq[k] : -4000);
+    for (int k = tid; k < kUMaxK; k += kUSplit) tb.w[k] = near_word(k < i ? eq[k].x : -4000);
     if (tid < kUN) {
       tb.g[tid] = -2147483647;
       tb.top[tid] = 0;
@@ -793,13 +823,24 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   __syncthreads();
   auto wprime = [&](int k, int c) -> double {
     const int gc = n0 + c;
-    if (k >= i || gc >= s || (upper && k > gc) || eq[k] < -2000) return 0.0;
-    return ldexp(W[k + static_cast<int64_t>(gc) * ldw], eq[k]);
+    if (k >= i || gc >= s || (upper && k > gc)) return 0.0;
+    const double wk = W[k + static_cast<int64_t>(gc) * ldw];
+    if (non_finite(wk)) return wk;
+    return eq[k].x < -2000 ? 0.0 : ldexp(wk, eq[k].x);
   };
   if (warp < kUWarps) {
     const int c = lane;
     double mx = 0.0;
-    for (int k = warp; k < i; k += kUWarps) mx = fmax(mx, fabs(wprime(k, c)));
+    for (int k = warp; k < i; k += kUWarps) {
+      const double wk = wprime(k, c);
+      if (non_finite(wk)) {
+        atomicMax(&tb.g[c], kUNonFinite);
+        sh.bad = 1;
+      } else {
+        mx = fmax(mx, fabs(wk));
+      }
+      if (eq[k].y > 0) sh.bad = 1;
+    }
     if (mx > 0.0) {
       int ee = 0;
       frexp(mx, &ee);
@@ -809,7 +850,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   __syncthreads();
   if (warp < kUWarps) {
     const int c = lane;
-    const int gc = tb.g[c] > -2000 ? tb.g[c] : -4000;
+    const int gc = tb.g[c] > -2000 && tb.g[c] != kUNonFinite ? tb.g[c] : -4000;
     for (int k = warp; k < i; k += kUWarps) {
       const double wk = wprime(k, c);
       uint32_t w8[kDig];
@@ -959,7 +1000,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           if (eout) {
             // the output column's exponent for the products that follow
             uint32_t t = static_cast<uint32_t>(__double2hiint(p)) & 0x7FFFFFFFu;
-            if (r >= n || t >= 0x7FF00000u) t = 0;
+            if (r >= n) t = 0;
             t = __reduce_max_sync(0xffffffffu, t);
             if (lane == 0) atomicMax(&tb.top[cg * kCols + cc], t);
           }
@@ -1008,7 +1049,7 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         }
         auto cut = [&](auto near) {
           constexpr bool kNear = decltype(near)::value;
-          auto ex = [&](int c) { return k0 + c < i ? __ldg(eq + k0 + c) : -4000; };
+          auto ex = [&](int c) { return k0 + c < i ? eq[k0 + c].x : -4000; };
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             uint32_t words[kDig][2];
@@ -1050,9 +1091,17 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   __syncthreads();
   if (sh.fail && tid == 0) atomicExch(err, 1);
   // (columns of zeros and subnormals keep the start value, as the cut takes
-  // both for zero)
-  if (eout && tid < kUN && n0 + tid < s && tb.top[tid] >= 0x00100000u)
-    atomicMax(eout + n0 + tid, static_cast<int>(tb.top[tid] >> 20) - 1022);
+  // both for zero; one that holds an Inf or a NaN gets the largest exponent)
+  if (eout && tid < kUN && n0 + tid < s && tb.top[tid] >= 0x00100000u) {
+    atomicMax(&eout[n0 + tid].x, min(static_cast<int>(tb.top[tid] >> 20) - 1022, 1024));
+    if (tb.top[tid] >= 0x7FF00000u) eout[n0 + tid].y = 1;
+  }
+  // A row of Q that holds an Inf or a NaN gives a row of NaN, a column of W'
+  // that holds one a column; the sums above have taken them for zeros.  Known
+  // from the exponents before the first tile and done after the last, so that
+  // finite operands pay one test (looking in the cut took 3 % of the update).
+  if (sh.bad && !sh.fail)
+    update_non_finite(n, i, s, Q, ldq, X, ldx, n0, g0, G, tb.g, eout);
   if (warp == 0) {
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1062,47 +1111,56 @@ oz_update_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   }
 }
 
-// e[c] = the exponent of column c's largest magnitude (|x| < 2^e): CTA
-// (c, z) takes rows [z rows, (z+1) rows) and merges its exponent with
-// atomicMax into e[c], which starts at a large negative value (all-zero
-// columns keep it).
+// e[c].x = the exponent of column c's largest finite magnitude (|x| < 2^e):
+// CTA (c, z) takes rows [z rows, (z+1) rows) and merges its exponent with
+// atomicMax into e[c].x, which starts at a large negative value (all-zero
+// columns keep it), as e[c].y does, which becomes 1 with an Inf or a NaN.
 __global__ void __launch_bounds__(256)
 col_exponent_kernel(int64_t n, const double* __restrict__ X, int64_t ld, int64_t rows,
-                    int* __restrict__ e) {
+                    int2* __restrict__ e) {
   // The largest |x| is found in integer arithmetic (the FP64 pipe would
   // bound this kernel far below HBM speed): for finite doubles, |x| orders
-  // like its bit pattern with the sign cleared.  NaNs (patterns above that
-  // of infinity) are skipped, as fmax would skip them.
+  // like its bit pattern with the sign cleared, and infinities and NaN have
+  // the patterns from that of infinity on.
   const uint64_t* col = reinterpret_cast<const uint64_t*>(X + static_cast<int64_t>(blockIdx.x) * ld);
   const int64_t r0 = static_cast<int64_t>(blockIdx.y) * rows;
   const int64_t r1 = (r0 + rows < n) ? r0 + rows : n;
   constexpr uint64_t kMag = 0x7FFFFFFFFFFFFFFFull, kInf = 0x7FF0000000000000ull;
-  auto take = [&](uint64_t& mx, uint64_t b) {
-    b &= kMag;
-    if (b <= kInf && b > mx) mx = b;
-  };
-  uint64_t mx = 0;
-  int64_t r = r0;
-  // one element to reach a 16-byte boundary, pairs with four loads in
-  // flight per thread, one element of tail
-  if ((reinterpret_cast<uintptr_t>(col + r) & 15) && r < r1) {
-    if (threadIdx.x == 0) take(mx, __ldg(col + r));
-    ++r;
-  }
-  const ulonglong2* pr = reinterpret_cast<const ulonglong2*>(col + r);
-  const int64_t np = (r1 - r) / 2;
-  for (int64_t p = threadIdx.x; p < np; p += 4 * 256) {
-    ulonglong2 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      v[u] = (p + u * 256 < np) ? __ldg(pr + p + u * 256) : make_ulonglong2(0, 0);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      take(mx, v[u].x);
-      take(mx, v[u].y);
+  // the largest pattern below `limit` of this thread's elements
+  auto largest = [&](uint64_t limit) {
+    uint64_t mx = 0;
+    auto take = [&](uint64_t b) {
+      b &= kMag;
+      if (b > mx && b < limit) mx = b;
+    };
+    int64_t r = r0;
+    // one element to reach a 16-byte boundary, pairs with four loads in
+    // flight per thread, one element of tail
+    if ((reinterpret_cast<uintptr_t>(col + r) & 15) && r < r1) {
+      if (threadIdx.x == 0) take(__ldg(col + r));
+      ++r;
     }
+    const ulonglong2* pr = reinterpret_cast<const ulonglong2*>(col + r);
+    const int64_t np = (r1 - r) / 2;
+    for (int64_t p = threadIdx.x; p < np; p += 4 * 256) {
+      ulonglong2 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        v[u] = (p + u * 256 < np) ? __ldg(pr + p + u * 256) : make_ulonglong2(0, 0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        take(v[u].x);
+        take(v[u].y);
+      }
+    }
+    if (((r1 - r) & 1) && threadIdx.x == 0) take(__ldg(col + r1 - 1));
+    return mx;
+  };
+  uint64_t mx = largest(~uint64_t(0));
+  if (mx >= kInf) {
+    e[blockIdx.x].y = 1;
+    mx = largest(kInf);
   }
-  if (((r1 - r) & 1) && threadIdx.x == 0) take(mx, __ldg(col + r1 - 1));
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const uint64_t o = __shfl_xor_sync(0xffffffffu, mx, off);
@@ -1118,13 +1176,13 @@ col_exponent_kernel(int64_t n, const double* __restrict__ X, int64_t ld, int64_t
     if (tb != 0) {
       int ee = 0;
       frexp(t, &ee);   // t = f 2^ee, f in [0.5, 1): |x| <= t < 2^ee
-      atomicMax(e + blockIdx.x, ee);
+      atomicMax(&e[blockIdx.x].x, ee);
     }
   }
 }
 
-void col_exponents(int64_t n, const double* X, int64_t ld, int cols, int* e, cudaStream_t st) {
-  SG_CUDA(cudaMemsetAsync(e, 0x80, sizeof(int) * cols, st));   // 0x80808080: no entry yet
+void col_exponents(int64_t n, const double* X, int64_t ld, int cols, int2* e, cudaStream_t st) {
+  SG_CUDA(cudaMemsetAsync(e, 0x80, sizeof(int2) * cols, st));   // 0x80808080: no entry yet
   int64_t z = static_cast<int64_t>(device_sm_count()) * 8 / cols;
   const int64_t zmax = (n + 4095) / 4096;
   if (z > zmax) z = zmax;
@@ -1137,8 +1195,8 @@ void col_exponents(int64_t n, const double* X, int64_t ld, int cols, int* e, cud
 
 // The exponents of a matrix's columns: those that the caller keeps, completed,
 // or all of them, in `scratch`.
-const int* exponents_of(int64_t n, const double* X, int64_t ld, int cols, ColExps* kept,
-                        int* scratch, cudaStream_t st) {
+const int2* exponents_of(int64_t n, const double* X, int64_t ld, int cols, ColExps* kept,
+                         int2* scratch, cudaStream_t st) {
   if (!kept) {
     col_exponents(n, X, ld, cols, scratch, st);
     return scratch;
@@ -1795,7 +1853,7 @@ int64_t oz_dot_part_size(int64_t n, int i, int s) {
   return oz_splits(n, i, s, nullptr) * i * s;
 }
 
-int64_t oz_exp_ints(int i, int s) { return static_cast<int64_t>(i) + s; }
+int64_t oz_exp_doubles(int i, int s) { return static_cast<int64_t>(i) + s; }
 
 bool oz_update_supported(int64_t n, const double* Q, int64_t ldq, int i, const double* X,
                          int64_t ldx, int s) {
@@ -1836,12 +1894,12 @@ bool oz_update_pays(int64_t n, int i, int s, bool upper) {
 }
 
 void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, int ldw,
-               double* X, int64_t ldx, int s, double alpha, double beta, bool upper, int* exps,
+               double* X, int64_t ldx, int s, double alpha, double beta, bool upper, int2* exps,
                cudaStream_t st, ColExps* eq, ColExps* ex) {
   int* err = oz_err_flag();
-  const int* e = exponents_of(n, Q, ldq, i, eq, exps, st);
+  const int2* e = exponents_of(n, Q, ldq, i, eq, exps, st);
   if (ex) {
-    SG_CUDA(cudaMemsetAsync(ex->e, 0x80, sizeof(int) * s, st));   // as col_exponents starts
+    SG_CUDA(cudaMemsetAsync(ex->e, 0x80, sizeof(int2) * s, st));   // as col_exponents starts
     ex->valid = s;
   }
   CUtensorMap mq, mx;
@@ -1852,7 +1910,8 @@ void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, 
   const int64_t ntiles = (n + kUM - 1) / kUM;
   const int64_t P = std::max<int64_t>(ct, std::min<int64_t>(device_sm_count(), ct * ntiles));
   oz_update_kernel<<<static_cast<unsigned>(P), kUThreads, oz_update_smem(i), st>>>(
-      mq, mx, n, i, s, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0, e, ex ? ex->e : nullptr, err);
+      mq, mx, n, i, s, W, ldw, X, ldx, alpha, beta, upper ? 1 : 0, e, ex ? ex->e : nullptr, Q, ldq,
+      err);
   SG_LAUNCH_CHECK();
   oz_check_error_pending.fetch_add(1);
 }
@@ -1878,15 +1937,17 @@ void oz_check_error(cudaStream_t st) {
 }
 
 void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int64_t ldx,
-            int s, int* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st,
-            ColExps* ceq, ColExps* cex) {
+            int s, int2* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st,
+            ColExps* ceq, ColExps* cex, const int2** feq, const int2** fex) {
   int* err = oz_err_flag();
   int64_t rows = 0;
   const int64_t S = oz_splits(n, i, s, &rows);
   SG_REQUIRE(S * i * s <= part_cap, SG_EINVAL, "oz_dot: workspace too small");
-  const int* eq = exponents_of(n, Q, ldq, i, ceq, exps, st);
-  const int* ex = X == Q && ldx == ldq && s <= i ? eq
-                                                 : exponents_of(n, X, ldx, s, cex, exps + i, st);
+  const int2* eq = exponents_of(n, Q, ldq, i, ceq, exps, st);
+  const int2* ex = X == Q && ldx == ldq && s <= i ? eq
+                                                  : exponents_of(n, X, ldx, s, cex, exps + i, st);
+  *feq = eq;
+  *fex = ex;
   CUtensorMap mq, mx;
   SG_REQUIRE(make_map64(&mq, Q, n, i, ldq, kOM) && make_map64(&mx, X, n, s, ldx, kON), SG_ECUDA,
              "cuTensorMapEncodeTiled failed");

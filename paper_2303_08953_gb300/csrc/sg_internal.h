@@ -163,13 +163,14 @@ void axpy_f32_to_f64(int64_t n, double alpha, const float* d, double* x,
                      cudaStream_t st);
 void fill_zero(int64_t n, double* x, cudaStream_t st);
 
-// Exponents of the columns of an FP64 matrix (|x| < 2^e, as the tensor-core
-// products need them) that the caller keeps beside it: device ints e, of
-// which the first `valid` hold.  block_dot and block_update complete them
-// where they need them and set those of the columns that they write; whoever
-// else writes the columns sets valid to 0.
+// Exponents of the columns of an FP64 matrix (of its finite values, |x| < 2^e,
+// as the tensor-core products need them; .y > 0 where the column also holds
+// an Inf or a NaN) that the caller keeps beside it: device pairs e, of which
+// the first `valid` hold.  block_dot and block_update complete them where
+// they need them and set those of the columns that they write; whoever else
+// writes the columns sets valid to 0.
 struct ColExps {
-  int* e = nullptr;
+  int2* e = nullptr;
   int valid = 0;
 };
 
@@ -229,26 +230,27 @@ void tc_fetch_error(int* host, cudaStream_t st);
 void tc_report_error(int host, cudaStream_t st);
 // Tensor-core (tcgen05, TMA) FP64 block dot W = Q^T X from exact 8-bit
 // digit slices of both operands: split partials into `part` (part_cap
-// doubles), column exponents into `exps` (oz_exp_ints(i, s) ints), number of
+// doubles), column exponents into `exps` (i + s pairs, oz_exp_doubles(i, s)
+// doubles) or kept ones, those used in *feq and *fex (the reduction of the
+// partials gives NaN for their non-finite columns), number of
 // splits in *nsplit; a bounded wait that ran out sets a device flag that
 // oz_check_error reads (and clears, then throws).
 bool oz_dot_supported(int64_t n, const double* Q, int64_t ldq, int i, const double* X,
                       int64_t ldx, int s);
 int64_t oz_dot_part_size(int64_t n, int i, int s);
-int64_t oz_exp_ints(int i, int s);
+int64_t oz_exp_doubles(int i, int s);
 bool oz_dot_pays(int64_t n, int i, int s, bool sym);
 // Tensor-core FP64 block update X = beta X + alpha Q W (W on the device, i x s,
-// upper-triangular if `upper`), from the same digit slices; exps: i ints.
+// upper-triangular if `upper`), from the same digit slices; exps: i pairs.
 bool oz_update_supported(int64_t n, const double* Q, int64_t ldq, int i, const double* X,
                          int64_t ldx, int s);
 bool oz_update_pays(int64_t n, int i, int s, bool upper);
 void oz_update(int64_t n, const double* Q, int64_t ldq, int i, const double* W, int ldw,
-               double* X, int64_t ldx, int s, double alpha, double beta, bool upper, int* exps,
-               cudaStream_t st,
-               ColExps* eq, ColExps* ex);
+               double* X, int64_t ldx, int s, double alpha, double beta, bool upper, int2* exps,
+               cudaStream_t st, ColExps* eq, ColExps* ex);
 void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int64_t ldx,
-            int s, int* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st,
-            ColExps* eq, ColExps* ex);
+            int s, int2* exps, double* part, int64_t part_cap, int* nsplit, cudaStream_t st,
+            ColExps* eq, ColExps* ex, const int2** feq, const int2** fex);
 void oz_check_error(cudaStream_t st);
 void oz_fetch_error(int* host, cudaStream_t st);
 void oz_report_error(int host, cudaStream_t st);

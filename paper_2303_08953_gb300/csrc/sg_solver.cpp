@@ -47,7 +47,7 @@ Slots slots_for(int m, int k) {
   s.scal = o; o += 16;        // scalars (norms)
   s.H = o;    o += kk * kk;   // Arnoldi pre-pass Hessenberg ((k+1) x k)
   s.wn = o;   o += kk;        // pre-pass norms before projection
-  s.E = o;    o += (mm + 2 * kk + 1) / 2;   // column exponents (ints): Q, V, Y
+  s.E = o;    o += mm + 2 * kk;   // column exponents (pairs of ints): Q, V, Y
   s.total = o;
   return s;
 }
@@ -443,7 +443,7 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
   // column of Q keeps its own through the cycle and the updates give those of
   // what they write, so that only the powers are read for them (reading every
   // operand of every product took 8 % of the 128^3 FP64 solve).
-  int* exps = reinterpret_cast<int*>(h->small + sl.E);
+  int2* exps = reinterpret_cast<int2*>(h->small + sl.E);
   ColExps eQ{exps, 0}, eX{exps + h->ws_m + 1, 0}, eY{exps + h->ws_m + h->ws_k + 2, 0};
   const int max_iters = o.max_iters > 0 ? o.max_iters : 50 * m;
 
