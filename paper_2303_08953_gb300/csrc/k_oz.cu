@@ -1922,10 +1922,8 @@ void oz_fetch_error(int* host, cudaStream_t st) {
   SG_CUDA(cudaMemcpyAsync(host, oz_err_flag(), sizeof(int), cudaMemcpyDeviceToHost, st));
 }
 
-void oz_report_error(int host, cudaStream_t st) {
-  if (!host) return;
+void oz_clear_error(cudaStream_t st) {
   SG_CUDA(cudaMemsetAsync(oz_err_flag(), 0, sizeof(int), st));
-  throw Error(SG_ECUDA, "tensor-core FP64 block dot: a bounded wait ran out");
 }
 
 void oz_check_error(cudaStream_t st) {
@@ -1933,7 +1931,9 @@ void oz_check_error(cudaStream_t st) {
   int host = 0;
   oz_fetch_error(&host, st);
   SG_CUDA(cudaStreamSynchronize(st));
-  oz_report_error(host, st);
+  if (!host) return;
+  oz_clear_error(st);
+  throw Error(SG_ECUDA, "tensor-core FP64 block dot: a bounded wait ran out");
 }
 
 void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int64_t ldx,

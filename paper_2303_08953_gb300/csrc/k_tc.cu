@@ -410,10 +410,8 @@ void tc_fetch_error(int* host, cudaStream_t st) {
   SG_CUDA(cudaMemcpyAsync(host, tc_err_flag(), sizeof(int), cudaMemcpyDeviceToHost, st));
 }
 
-void tc_report_error(int host, cudaStream_t st) {
-  if (!host) return;
+void tc_clear_error(cudaStream_t st) {
   SG_CUDA(cudaMemsetAsync(tc_err_flag(), 0, sizeof(int), st));
-  throw Error(SG_ECUDA, "tensor-core block dot: a bounded wait ran out");
 }
 
 void tc_check_error(cudaStream_t st) {
@@ -421,7 +419,9 @@ void tc_check_error(cudaStream_t st) {
   int host = 0;
   tc_fetch_error(&host, st);
   SG_CUDA(cudaStreamSynchronize(st));
-  tc_report_error(host, st);
+  if (!host) return;
+  tc_clear_error(st);
+  throw Error(SG_ECUDA, "tensor-core block dot: a bounded wait ran out");
 }
 
 void tc_dot(int64_t n, const float* Q, int64_t ldq, int i, const float* X, int64_t ldx,

@@ -458,10 +458,8 @@ void tc_update_fetch_error(int* host, cudaStream_t st) {
   SG_CUDA(cudaMemcpyAsync(host, err_flag(), sizeof(int), cudaMemcpyDeviceToHost, st));
 }
 
-void tc_update_report_error(int host, cudaStream_t st) {
-  if (!host) return;
+void tc_update_clear_error(cudaStream_t st) {
   SG_CUDA(cudaMemsetAsync(err_flag(), 0, sizeof(int), st));
-  throw Error(SG_ECUDA, "tensor-core block update: a bounded wait ran out");
 }
 
 void tc_update_check_error(cudaStream_t st) {
@@ -469,7 +467,9 @@ void tc_update_check_error(cudaStream_t st) {
   int host = 0;
   tc_update_fetch_error(&host, st);
   SG_CUDA(cudaStreamSynchronize(st));
-  tc_update_report_error(host, st);
+  if (!host) return;
+  tc_update_clear_error(st);
+  throw Error(SG_ECUDA, "tensor-core block update: a bounded wait ran out");
 }
 
 }  // namespace sg

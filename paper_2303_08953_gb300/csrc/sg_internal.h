@@ -224,10 +224,10 @@ void tc_dot(int64_t n, const float* Q, int64_t ldq, int i, const float* X,
 void tc_check_error(cudaStream_t st);
 // The same in two halves, for a caller that synchronises anyway: fetch_error
 // queues the flag's copy to `host` (pinned; set to 0 at once where no kernel
-// has run since the last check), report_error, after the synchronisation,
-// throws on a flag that was set.
+// has run since the last check); after the synchronisation the caller clears
+// every flag that was set (clear_error) and throws (sg_timeouts.h).
 void tc_fetch_error(int* host, cudaStream_t st);
-void tc_report_error(int host, cudaStream_t st);
+void tc_clear_error(cudaStream_t st);
 // Tensor-core (tcgen05, TMA) FP64 block dot W = Q^T X from exact 8-bit
 // digit slices of both operands: split partials into `part` (part_cap
 // doubles), column exponents into `exps` (i + s pairs, oz_exp_doubles(i, s)
@@ -253,7 +253,7 @@ void oz_dot(int64_t n, const double* Q, int64_t ldq, int i, const double* X, int
             ColExps* eq, ColExps* ex, const int2** feq, const int2** fex);
 void oz_check_error(cudaStream_t st);
 void oz_fetch_error(int* host, cudaStream_t st);
-void oz_report_error(int host, cudaStream_t st);
+void oz_clear_error(cudaStream_t st);
 // Tensor-core FP32 Gram G = X^T X (s <= 128 columns) from exact digit
 // slices: split partials of the upper triangle (entry (m, n), m <= n, at
 // m + n s) into `part`, column exponents into `exps` (s ints); a bounded
@@ -273,7 +273,7 @@ void tc_update(int64_t n, const float* Q, int64_t ldq, int i, const double* W,
                cudaStream_t st);
 void tc_update_check_error(cudaStream_t st);
 void tc_update_fetch_error(int* host, cudaStream_t st);
-void tc_update_report_error(int host, cudaStream_t st);
+void tc_update_clear_error(cudaStream_t st);
 
 // dst[k] = src[idx[k]], k < count (device arrays).
 // Structure checks of a square CSR matrix on the device (synchronises):

@@ -5,6 +5,7 @@
 // host twice per block (after each Gram matrix), carrying (i+s) x s
 // values.
 #include "sg_solver.h"
+#include "sg_timeouts.h"
 
 #include <algorithm>
 #include <chrono>
@@ -467,11 +468,13 @@ void solve_impl(sg_handle* h, const DevCsr& M, const SolveOpts& o,
     }
   };
   auto report_errors = [&] {
-    oz_report_error(flags[0], st);
-    if (sizeof(T) == 4) {
-      tc_report_error(flags[1], st);
-      tc_update_report_error(flags[2], st);
-    }
+    const char* const names[3] = {"digit-slice products", "block dot", "block update"};
+    const std::string who = collect_timeouts(flags, names, sizeof(T) == 4 ? 3 : 1, [&](int k) {
+      if (k == 0) oz_clear_error(st);
+      else if (k == 1) tc_clear_error(st);
+      else tc_update_clear_error(st);
+    });
+    if (!who.empty()) throw Error(SG_ECUDA, "tensor-core " + who + ": a bounded wait ran out");
   };
 
   // r = b - A x0, beta0 (Alg. 4, first line)
