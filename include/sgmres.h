@@ -190,8 +190,10 @@ sg_status sg_update_values(sg_handle* h, const double* val,
 
 /* Storage the SpMV kernels use for the analysed matrix: *sell = 1 when
  * the SELL-32 copy (slices of 32 rows, column-major within a slice) was
- * built at ingest, 0 when the CSR arrays are walked directly (the padding
- * to each slice's longest row would exceed 20% of nnz); *stored = the
+ * built at ingest (rows in order, or sorted by length within windows of 1024
+ * rows where that pads too much), 0 when the CSR arrays are walked directly
+ * (the padding to each slice's longest row would exceed 20% of nnz plus 32
+ * entries a slice either way); *stored = the
  * entries the SpMV reads per product (padded count for SELL-32, nnz for
  * CSR).  Either pointer may be NULL.  Not in the paper: a layout report.
  * Errors: SG_EINVAL (NULL handle), SG_ESTATE (no matrix). */
