@@ -92,3 +92,58 @@ def test_a_pattern_that_ends_in_csr_costs_one_kernel(solver):
     ln = _lengths("a long row in 64", n)
     assert launches(_matrix(ln)) == checks + 1
     assert not solver.matrix_info()[0]
+
+
+def _uneven_diagonal(n, seed):
+    """Uneven rows with a dominant diagonal (sorted windows), columns sorted."""
+    rng = np.random.default_rng(seed)
+    ln = rng.integers(3, 30, n)
+    ptr = np.zeros(n + 1, np.int64)
+    np.cumsum(ln, out=ptr[1:])
+    cols = np.concatenate([np.sort(np.append(i, rng.choice(np.delete(np.arange(max(0, i - 60),
+                           min(n, i + 61)), min(i, 60)), l - 1, replace=False)))
+                           for i, l in zip(range(n), ln)])
+    vals = rng.uniform(-1.0, 1.0, ptr[-1])
+    rows = np.repeat(np.arange(n), ln)
+    vals[cols == rows] = 1.5 * ln
+    return W.CSR(n, ptr.astype(np.int32), cols.astype(np.int32), vals)
+
+
+def test_sorted_rows_with_column_equilibration(solver):
+    """A D_c shares A's row order: the solution to 1e-11 of the residual, for
+    columns of sizes up to 2^12 apart (diagonally dominant rows, so x is
+    within 1e-9 of the one b was formed from)."""
+    A = _uneven_diagonal(4133, 1)
+    d = 2.0 ** np.random.default_rng(2).integers(0, 13, A.n)
+    A = W.CSR(A.n, A.rowptr, A.colind, A.val * d[A.colind])
+    rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
+    x = np.random.default_rng(3).uniform(-1, 1, A.n) / d
+    b = np.bincount(rows, A.val * x[A.colind], minlength=A.n)
+    solver.analyze_csr(A)
+    sell, stored = solver.matrix_info()
+    in_order = _slices(np.diff(A.rowptr))
+    assert sell and stored < in_order
+    got, info = solver.solve(torch.as_tensor(b, device="cuda:0"), m=60, s=6, tol=1e-12,
+                             equilibrate="column")
+    assert info.converged
+    assert np.linalg.norm((got.cpu().numpy() - x) * d) <= 1e-9 * np.linalg.norm(x * d)
+
+
+def test_sorted_rows_of_a_row_block(solver):
+    """A row block in local numbering (more columns than rows, unsorted)."""
+    A = _uneven_diagonal(3000, 4)
+    lo, hi = 500, 2600
+    p, q = A.rowptr[lo], A.rowptr[hi]
+    rp = (A.rowptr[lo:hi + 1] - p).astype(np.int32)
+    local, halo = sg.halo_plan(rp, A.colind[p:q], lo, hi)
+    solver.analyze_rows(rp, local, A.val[p:q], hi - lo + halo.size)
+    x = np.random.default_rng(5).standard_normal(A.n)
+    xl = np.concatenate([x[lo:hi], x[halo]])
+    y = solver.spmv_newton(torch.as_tensor(xl, device="cuda:0"), theta=0.5, gamma=2.0)
+    rows = np.repeat(np.arange(hi - lo), np.diff(rp))
+    prod = A.val[p:q] * x[A.colind[p:q]]
+    ref = (np.bincount(rows, prod, minlength=hi - lo) - 0.5 * x[lo:hi]) / 2.0
+    mag = np.bincount(rows, np.abs(prod), minlength=hi - lo) + np.abs(x[lo:hi])
+    got = y.cpu().numpy()[:hi - lo]
+    assert np.all(np.abs(got - ref) <= 40 * 2.0 ** -53 * mag)
+    assert solver.matrix_info()[0]
