@@ -42,8 +42,8 @@
 //     output columns each.
 // A stage takes about 3,300 cycles: 2,200 the cut, 700 (a quarter of a
 // readout) the level sums, 400 waits; the MMAs' 1,800 overlap the cut.  At
-// 2^21 rows the 121 x 120 dot takes 3.61 ms with the exponents (4.27 before
-// the cut and the readout were shortened), the Gram of 120 3.30 ms (3.95).
+// 2^21 rows the 121 x 120 dot takes 3.45 ms with the exponents (4.27 before
+// the cut and the readout were shortened), the Gram of 120 3.15 ms (3.95).
 // Every wait is bounded: on timeout the kernel records an error, drains
 // its own copies, frees its tensor memory and returns.
 #include <cuda.h>
@@ -141,19 +141,17 @@ __device__ __forceinline__ uint2 biased62(double x, int e) {
 // The same for |x| in [2^(e - 32), 2^e), where the shift is 1 .. 31 (the
 // mantissa's top bit at bit 62 first), from the column's word
 // w = near_word(e): E + w is minus the shift modulo 32.  It needs neither the
-// clamps nor the test for E = 0 of the general form above.  (Written as
-// multiply-adds, which the compiler turns into shifts and additions where
-// they are cheaper; with factors it cannot see, all of it on the FMA pipe,
-// the kernels were 3 % slower.)
+// clamps nor the test for E = 0 of the general form above.  (The products are
+// C++ expressions: as multiply-adds in PTX the 121 x 120 dot at 2^21 rows
+// takes 3.57 ms instead of 3.45, the Gram of 120 3.28 instead of 3.15.)
 __device__ __forceinline__ uint2 biased62_near(uint32_t xh, uint32_t xl, uint32_t w, uint32_t one) {
   const uint32_t h = ((xh << 10) & 0x3FFFFFFFu) | 0x40000000u;
-  uint64_t m, sh, r;
-  asm("mad.wide.u32 %0, %1, 1024, %2;" : "=l"(m) : "r"(xl), "l"(static_cast<uint64_t>(h) << 32));
-  asm("mad.wide.u32 %0, %1, 4096, %2;" : "=l"(sh) : "r"(xh), "l"(static_cast<uint64_t>(w) << 32));
+  const uint64_t m = static_cast<uint64_t>(xl) * 1024u + (static_cast<uint64_t>(h) << 32);
+  const uint64_t sh = static_cast<uint64_t>(xh) * 4096u + (static_cast<uint64_t>(w) << 32);
   const uint32_t H = static_cast<uint32_t>(m >> 32), c = static_cast<uint32_t>(sh >> 32);
   const uint32_t lo = __funnelshift_l(static_cast<uint32_t>(m), H, c);
   const uint32_t hi = __funnelshift_l(H, 0u, c);
-  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(lo), "r"(one), "l"(0x8080808080808080ull));
+  const uint64_t r = static_cast<uint64_t>(lo) * one + 0x8080808080808080ull;
   return make_uint2(static_cast<uint32_t>(r), hi * one + static_cast<uint32_t>(r >> 32));
 }
 
@@ -667,9 +665,9 @@ oz_dot_kernel(const __grid_constant__ CUtensorMap mapQ,
 // What bounds it: the cut (about 2,200 of the 3,300 cycles of a stage; the
 // MMAs, eight of N = 256 .. 32 each 16 columns, take 1,800 and overlap it),
 // then the readout and the epilogue, which the MMAs wait for.  At 2^21 rows:
-// 121 x 120 4.69 ms (6.40 with the general cut, a level at a time and the
+// 121 x 120 4.59 ms (6.40 with the general cut, a level at a time and the
 // product with alpha on the FP64 pipe), the triangular product of 120
-// 3.96 ms (6.33; 5.30 of it from leaving out W's lower triangle).
+// 3.70 ms (6.33).
 constexpr int kUM = 128;
 constexpr int kUN = 32;
 constexpr int kUS = 32;                                 // columns of Q per stage

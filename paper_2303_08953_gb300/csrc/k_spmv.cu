@@ -658,8 +658,9 @@ __device__ __forceinline__ double fx_decode(long long code, double unit) {
   return static_cast<double>(x) * unit;
 }
 
-// a b + c.  In PTX: written in C++, the compiler forms a 64 x 64 bit product
-// of halves taken from a 64-bit word (three multiply-adds instead of one).
+// a b + c as the one multiply-add it is (with the C++ expression in its place
+// a 60-step pre-pass takes 14.97 ms instead of 14.15 at 2.10M rows, 4.67
+// instead of 4.66 at 149K).
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
   long long d;
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
