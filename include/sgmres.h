@@ -294,8 +294,10 @@ sg_status sg_block_update(sg_handle* h, int64_t n, const double* Q,
  * column's largest magnitude (every value within 2^23 of it exact; entry
  * (a, b) within 2^-46 (max|x_a| sum|x_b| + max|x_b| sum|x_a|)
  * + n 2^-58 max|x_a| max|x_b| of the exact Gram, plus one rounding); else
- * from exact FP32 products accumulated with compensated sums (accurate to
- * ~eps_32^2 relative to sum |x_k y_k|).  An Inf or a NaN in a column makes
+ * from exact FP32 products accumulated with compensated sums (largest error
+ * measured at 2^21 rows, relative to the product of the columns' norms:
+ * 6e-14 for normal entries, 3e-12 for columns of one large entry; 7e-16 and
+ * 2e-13 on the tensor cores).  An Inf or a NaN in a column makes
  * that column's row and column of the Gram non-finite (NaN on the tensor
  * cores).  Otherwise, when the
  * leading dimensions are multiples of

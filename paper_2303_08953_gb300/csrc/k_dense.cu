@@ -16,9 +16,10 @@
 // FP32 data: projections accumulate in FP32 per 32-row stage and fold the
 // stage sums into a compensated total; Gram matrices (EXACT) form every
 // product exactly (p = a b rounded plus its FMA remainder) and add it with
-// a two-sum, so the Gram of FP32 vectors is accurate to about eps_32^2
-// relative to the sum of |products| -- the accuracy the partial Cholesky
-// bound of the FP32 basis relies on.
+// a two-sum, so the Gram of FP32 vectors is accurate far beyond FP32 (largest
+// error measured at 2^21 rows, relative to the product of the columns'
+// norms: 6e-14 for normal entries, 3e-12 for columns of one large entry) --
+// what the partial Cholesky bound of the FP32 basis relies on.
 #include <algorithm>
 #include <atomic>
 #include <cstdlib>

@@ -753,8 +753,10 @@ void solve_fp32_ir(sg_handle* h, const DevCsr& M, const SolveOpts& o,
   // Bounds of the FP32 basis.  The paper's rule Omega ~ 0.1 eps^-1/2
   // (Sec. 3.2) is set by the accuracy of the Gram matrix the Cholesky
   // factor comes from; the FP32 Gram matrices here are formed from exact
-  // products with compensated sums (relative accuracy ~2^-40 after the
-  // split reduction), so Omega_32 = 0.1 (2^-40)^-1/2 = 0.1 2^20.  That also
+  // products with compensated sums or from digit slices (largest errors
+  // measured at 2^21 rows, relative to the columns' norms: 2^-44 and 2^-50
+  // for normal entries, 2^-38 and 2^-42 for columns of one large entry), so
+  // about 2^-40 and Omega_32 = 0.1 (2^-40)^-1/2 = 0.1 2^20.  That also
   // keeps the FP32 triangular product's orthogonality loss eps_32 Omega
   // below 1e-2, which the second CholQR pass removes.  The estimator uses
   // the basis round-off eps_32 = 2^-24 and the same threshold.
