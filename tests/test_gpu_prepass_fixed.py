@@ -137,24 +137,3 @@ def test_nan_in_the_matrix_reaches_h(solver):
     q = np.full(A.n, 1.0 / 40)
     H, steps = _run(solver, W.CSR(A.n, A.rowptr, A.colind, val), q, 4)
     assert steps == 1 and np.isnan(H[0, 0]) and np.isnan(H[1, 0])
-
-
-# A CTA's rows end inside a warp's batch: 1024-row CTAs hold 512 pairs of
-# rows, 4 pairs a thread and batch, so the last batch of the last CTA leaves
-# lanes of a warp idle for these row counts (and a whole batch precedes it
-# from 4096 rows a CTA on: 152 x 4096 rows and more)
-@pytest.mark.parametrize("n", [37, 101, 1024 + 75, 3 * 1024 + 333, 700_001, 1_400_321])
-def test_a_batch_that_ends_inside_a_warp(solver, n):
-    i = np.arange(n)
-    ptr = np.concatenate([[0], np.cumsum(np.where(i + 1 < n, 2, 1))]).astype(np.int32)
-    cols = np.empty(ptr[-1], np.int32)
-    vals = np.empty(ptr[-1])
-    cols[ptr[:-1]] = i
-    vals[ptr[:-1]] = 2.0 + (i % 7) / 7.0
-    cols[ptr[:-2] + 1] = i[1:]
-    vals[ptr[:-2] + 1] = -1.0
-    q = np.cos(0.37 * i) + 0.5
-    q /= np.linalg.norm(q)
-    A = W.CSR(n, ptr, cols, vals)
-    H, steps = _run(solver, A, q, 5)
-    _check(A, q, 5, H, steps)

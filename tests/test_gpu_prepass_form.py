@@ -136,3 +136,24 @@ def test_even_rows_whose_product_vanishes(solver):
     q /= np.linalg.norm(q)
     solver.analyze_csr(A)
     _check(A, q, k, *_arnoldi(solver, q, k))
+
+
+# A CTA's rows end inside a warp's batch: 1024-row CTAs hold 512 pairs of
+# rows, 4 pairs a thread and batch, so the last batch of the last CTA leaves
+# lanes of a warp idle for these row counts (and a whole batch precedes it
+# from 4096 rows a CTA on: 152 x 4096 rows and more)
+@pytest.mark.parametrize("n", [37, 101, 1024 + 75, 3 * 1024 + 333, 700_001, 1_400_321])
+def test_a_batch_that_ends_inside_a_warp(solver, n):
+    i = np.arange(n)
+    ptr = np.concatenate([[0], np.cumsum(np.where(i + 1 < n, 2, 1))]).astype(np.int32)
+    cols = np.empty(ptr[-1], np.int32)
+    vals = np.empty(ptr[-1])
+    cols[ptr[:-1]] = i
+    vals[ptr[:-1]] = 2.0 + (i % 7) / 7.0
+    cols[ptr[:-2] + 1] = i[1:]
+    vals[ptr[:-2] + 1] = -1.0
+    q = np.cos(0.37 * i) + 0.5
+    q /= np.linalg.norm(q)
+    A = W.CSR(n, ptr, cols, vals)
+    solver.analyze_csr(A)
+    _check(A, q, 5, *_arnoldi(solver, q, 5))
